@@ -82,6 +82,16 @@ int alloc(T** dst, size_t n) {
 
 inline unsigned nblocks(size_t threads, int bs = 256) { return (unsigned)((threads + bs - 1) / bs); }
 
+// Threads per block of the kernels without shared memory (FP64 reconstruction
+// and face kernels, RK stages).  They are bound by the FP64 pipe of each SM, so
+// what counts is how evenly the warps spread over the 152 SMs: a 16^3 P1 face
+// launch is 48 blocks of 256 threads (104 SMs idle) but 192 of 64.  Measured with
+// 256 / 128 / 64 / 32 threads, us per launch: P1 face at 16^3 32.6 / 20.6 / 20.2 /
+// 18.5, RK stage there 9.7 / 8.6 / 8.2 / 8.2, inviscid P2 face at 33 x 36 x 39 314 /
+// 304 / 304 / 304, P2 reconstruction at 72 x 80 x 88 2455 / 2435 / 2435 / 2434, its
+// RK stage 54.2 / 53.5 / 53.6 / 52.6, mixed RK stage at 96^3 53.8 / 52.4 / 52.4 / 55.2.
+constexpr int kFlatThreads = 64;
+
 enum {
   kKindRecon = 0,
   kKindFace = 1,
@@ -398,29 +408,29 @@ int launch_recon_raw(ucns_mesh* m, const double* U, cudaStream_t s) {
   a.lams = 1.0 / lsum;
   a.lamc = m->P.lambda_central;
   a.eps = m->P.epsilon;
-  const unsigned g = nblocks((size_t)m->N * 5);
+  const unsigned g = nblocks((size_t)m->N * 5, kFlatThreads);
   const bool gated = a.gate != nullptr;
   const bool walls = m->n_boundary > 0;
   if (m->K == 3)
-    k_recon<1, false, 6, false><<<g, 256, 0, s>>>(a);
+    k_recon<1, false, 6, false><<<g, kFlatThreads, 0, s>>>(a);
   else if (m->nd == 0)
-    k_recon<2, false, 6, false><<<g, 256, 0, s>>>(a);
+    k_recon<2, false, 6, false><<<g, kFlatThreads, 0, s>>>(a);
   else if (walls && m->nd == 6)
-    k_recon<2, true, 6, false, true><<<g, 256, 0, s>>>(a);
+    k_recon<2, true, 6, false, true><<<g, kFlatThreads, 0, s>>>(a);
   else if (walls && m->nd == 5)
-    k_recon<2, true, 5, false, true><<<g, 256, 0, s>>>(a);
+    k_recon<2, true, 5, false, true><<<g, kFlatThreads, 0, s>>>(a);
   else if (walls)
-    k_recon<2, true, 4, false, true><<<g, 256, 0, s>>>(a);
+    k_recon<2, true, 4, false, true><<<g, kFlatThreads, 0, s>>>(a);
   else if (m->nd == 5)
-    k_recon<2, true, 5, false><<<g, 256, 0, s>>>(a);
+    k_recon<2, true, 5, false><<<g, kFlatThreads, 0, s>>>(a);
   else if (m->nd == 6 && gated)
-    k_recon<2, true, 6, true><<<g, 256, 0, s>>>(a);
+    k_recon<2, true, 6, true><<<g, kFlatThreads, 0, s>>>(a);
   else if (m->nd == 6)
-    k_recon<2, true, 6, false><<<g, 256, 0, s>>>(a);
+    k_recon<2, true, 6, false><<<g, kFlatThreads, 0, s>>>(a);
   else if (gated)
-    k_recon<2, true, 4, true><<<g, 256, 0, s>>>(a);
+    k_recon<2, true, 4, true><<<g, kFlatThreads, 0, s>>>(a);
   else
-    k_recon<2, true, 4, false><<<g, 256, 0, s>>>(a);
+    k_recon<2, true, 4, false><<<g, kFlatThreads, 0, s>>>(a);
   UCNS_CUDA(cudaGetLastError());
   return UCNS_OK;
 }
@@ -441,16 +451,16 @@ int launch_face_raw(ucns_mesh* m, cudaStream_t s) {
   a.c = flux_const(m->P);
   for (int v = 0; v < 5; v++) a.uinf[v] = m->uinf[v];
   const bool visc = m->P.reynolds > 0.0;
-  const unsigned g = nblocks((size_t)m->F * m->nq);
+  const unsigned g = nblocks((size_t)m->F * m->nq, kFlatThreads);
   if (m->n_boundary > 0) {  // inviscid (checked at precompute)
-    if (m->K == 3) k_face<1, false, true><<<g, 256, 0, s>>>(a);
-    else k_face<2, false, true><<<g, 256, 0, s>>>(a);
+    if (m->K == 3) k_face<1, false, true><<<g, kFlatThreads, 0, s>>>(a);
+    else k_face<2, false, true><<<g, kFlatThreads, 0, s>>>(a);
   } else if (m->K == 3) {
-    if (visc) k_face<1, true><<<g, 256, 0, s>>>(a);
-    else k_face<1, false><<<g, 256, 0, s>>>(a);
+    if (visc) k_face<1, true><<<g, kFlatThreads, 0, s>>>(a);
+    else k_face<1, false><<<g, kFlatThreads, 0, s>>>(a);
   } else {
-    if (visc) k_face<2, true><<<g, 256, 0, s>>>(a);
-    else k_face<2, false><<<g, 256, 0, s>>>(a);
+    if (visc) k_face<2, true><<<g, kFlatThreads, 0, s>>>(a);
+    else k_face<2, false><<<g, kFlatThreads, 0, s>>>(a);
   }
   UCNS_CUDA(cudaGetLastError());
   return UCNS_OK;
@@ -473,16 +483,16 @@ int launch_rk_raw(ucns_mesh* m, int stage, const double* U0, const double* Us, d
   a.N = (int)m->N;
   a.F = (int)m->F;
   a.gm1 = m->P.gamma - 1.0;
-  const unsigned g = nblocks((size_t)m->N);
+  const unsigned g = nblocks((size_t)m->N, kFlatThreads);
 #define UCNS_RK(ST)                                                           \
   do {                                                                        \
     if (mixed(m)) {                                                           \
-      if (m->nfc == 6) k_rk<ST, 6, float><<<g, 256, 0, s>>>(a);               \
-      else k_rk<ST, 4, float><<<g, 256, 0, s>>>(a);                           \
+      if (m->nfc == 6) k_rk<ST, 6, float><<<g, kFlatThreads, 0, s>>>(a);               \
+      else k_rk<ST, 4, float><<<g, kFlatThreads, 0, s>>>(a);                           \
     } else {                                                                  \
-      if (m->nfc == 6) k_rk<ST, 6, double><<<g, 256, 0, s>>>(a);              \
-      else if (m->nfc == 5) k_rk<ST, 5, double><<<g, 256, 0, s>>>(a);         \
-      else k_rk<ST, 4, double><<<g, 256, 0, s>>>(a);                          \
+      if (m->nfc == 6) k_rk<ST, 6, double><<<g, kFlatThreads, 0, s>>>(a);              \
+      else if (m->nfc == 5) k_rk<ST, 5, double><<<g, kFlatThreads, 0, s>>>(a);         \
+      else k_rk<ST, 4, double><<<g, kFlatThreads, 0, s>>>(a);                          \
     }                                                                         \
   } while (0)
   switch (stage) {
@@ -513,16 +523,16 @@ int launch_rk54_raw(ucns_mesh* m, int stage, const double* U0, const double* Us,
   a.N = (int)m->N;
   a.F = (int)m->F;
   a.gm1 = m->P.gamma - 1.0;
-  const unsigned g = nblocks((size_t)m->N);
+  const unsigned g = nblocks((size_t)m->N, kFlatThreads);
 #define UCNS_RK54(ST)                                                         \
   do {                                                                        \
     if (mixed(m)) {                                                           \
-      if (m->nfc == 6) k_rk54<ST, 6, float><<<g, 256, 0, s>>>(a);             \
-      else k_rk54<ST, 4, float><<<g, 256, 0, s>>>(a);                         \
+      if (m->nfc == 6) k_rk54<ST, 6, float><<<g, kFlatThreads, 0, s>>>(a);             \
+      else k_rk54<ST, 4, float><<<g, kFlatThreads, 0, s>>>(a);                         \
     } else {                                                                  \
-      if (m->nfc == 6) k_rk54<ST, 6, double><<<g, 256, 0, s>>>(a);            \
-      else if (m->nfc == 5) k_rk54<ST, 5, double><<<g, 256, 0, s>>>(a);       \
-      else k_rk54<ST, 4, double><<<g, 256, 0, s>>>(a);                        \
+      if (m->nfc == 6) k_rk54<ST, 6, double><<<g, kFlatThreads, 0, s>>>(a);            \
+      else if (m->nfc == 5) k_rk54<ST, 5, double><<<g, kFlatThreads, 0, s>>>(a);       \
+      else k_rk54<ST, 4, double><<<g, kFlatThreads, 0, s>>>(a);                        \
     }                                                                         \
   } while (0)
   switch (stage) {
@@ -698,7 +708,7 @@ int diag_sums_into(ucns_mesh* m, const double* U, double* out, cudaStream_t s) {
                                                              (int)m->N, m->d.red);
   else
     k_diag_partial<double><<<m->d.red_blocks, kRedThreads, 0, s>>>(U, m->d.coef, m->d.vol, (int)m->N, m->d.red);
-  k_diag_final<<<1, 32, 0, s>>>(m->d.red, m->d.red_blocks, out);
+  k_sum_partials<<<1, 32 * 4, 0, s>>>(m->d.red, m->d.red_blocks, 4, 4, out);
   UCNS_CUDA(cudaGetLastError());
   return UCNS_OK;
 }
@@ -737,7 +747,7 @@ int gate_check(ucns_mesh* m, const double* U, double* rel, cudaStream_t s, int s
     int r = diag_sums_into(m, U, sums + 4, s);
     if (r) return r;
     k_ke_rate_partial<<<m->d.red_blocks, 256, 0, s>>>(U, m->gate_R, m->gate_R + n5, m->d.vol, (int)m->N, m->d.red);
-    k_sum_partials<<<1, 32, 0, s>>>(m->d.red, m->d.red_blocks, kRedStride, kKeRateSums, sums + 8);
+    k_sum_partials<<<1, 32 * kKeRateSums, 0, s>>>(m->d.red, m->d.red_blocks, kRedStride, kKeRateSums, sums + 8);
     UCNS_CUDA(cudaGetLastError());
     return launch_dt_to(m, U, sums + 13, s);  // the CFL time step of U, apart from the solver's own
   });
@@ -1296,7 +1306,7 @@ int ucns_diagnostics(ucns_mesh* m, const double* U, ucns_diag* out, void* stream
     else
       k_diag_partial<double><<<m->d.red_blocks, kRedThreads, 0, s>>>(U, m->d.coef, m->d.vol, (int)m->N, m->d.red);
     // the final sums land in the first 4 doubles of G (free between residuals)
-    k_diag_final<<<1, 32, 0, s>>>(m->d.red, m->d.red_blocks, m->d.G);
+    k_sum_partials<<<1, 32 * 4, 0, s>>>(m->d.red, m->d.red_blocks, 4, 4, m->d.G);
     UCNS_CUDA(cudaGetLastError());
     return UCNS_OK;
   });

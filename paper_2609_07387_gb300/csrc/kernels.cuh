@@ -876,12 +876,21 @@ __global__ void __launch_bounds__(kRedThreads)
     for (int q = 0; q < 4; q++) part[(size_t)blockIdx.x * 4 + q] = sm[q][0];
 }
 
-__global__ void k_diag_final(const double* __restrict__ part, int nb, double* __restrict__ out) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  double s[4] = {0, 0, 0, 0};
-  for (int b = 0; b < nb; b++)
-    for (int q = 0; q < 4; q++) s[q] += part[(size_t)b * 4 + q];
-  for (int q = 0; q < 4; q++) out[q] = s[q];
+// out[q] = sum of part[stride b + q] over the nb blocks, q < nq <= 8: one warp
+// per sum, each lane adding every 32nd partial in block order, then a fixed
+// shuffle tree (deterministic).  Launched as one block of 32 nq threads.  Bound
+// by latency: one thread adding them in turn took 146 us for four sums of 608
+// partials (a dependent load per addition); with k_diag_partial the diagnostics
+// at 16^3 went from 120 to 17 us.
+__global__ void __launch_bounds__(256) k_sum_partials(const double* __restrict__ part, int nb, int stride, int nq,
+                                                      double* __restrict__ out) {
+  const int q = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (q >= nq) return;
+  double s = 0.0;
+  for (int b = lane; b < nb; b += 32) s += part[(size_t)b * stride + q];
+#pragma unroll
+  for (int off = 16; off >= 1; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
+  if (lane == 0) out[q] = s;
 }
 
 // ALU throughput probes: kPeakChains independent FMA chains per thread (the

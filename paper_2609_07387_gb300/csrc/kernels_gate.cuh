@@ -242,14 +242,4 @@ __global__ void __launch_bounds__(256) k_ke_rate_partial(const double* __restric
     for (int q = 0; q < kKeRateSums; q++) part[(size_t)blockIdx.x * kRedStride + q] = sm[q][0];
 }
 
-// out[q] = sum over blocks, in block order, of part[stride b + q], q < nq
-__global__ void k_sum_partials(const double* __restrict__ part, int nb, int stride, int nq, double* __restrict__ out) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  for (int q = 0; q < nq; q++) {
-    double s = 0.0;
-    for (int b = 0; b < nb; b++) s += part[(size_t)b * stride + q];
-    out[q] = s;
-  }
-}
-
 }  // namespace ucns
