@@ -73,6 +73,45 @@ int upload_blocked(T** dst, const std::vector<S>& src, int rows, int64_t N, bool
   return upload(dst, b);
 }
 
+// Rows k < K of cell i's least-squares matrix src [K][M][N] as limb pairs P and
+// exponents E, entry (k, m) at P[(k M + m) TC + c] (fixed.cuh)
+void fixed_rows(const double* src, int K, int M, int64_t N, int64_t i, int TC, int c, int2* P, int16_t* E) {
+  for (int k = 0; k < K; k++) {
+    double l1 = 0.0;
+    for (int m = 0; m < M; m++) l1 += std::fabs(src[((size_t)k * M + m) * N + i]);
+    const int e = fx_row_exponent(l1);
+    E[k * TC + c] = (int16_t)e;
+    const double up = std::ldexp(1.0, std::min(60 - e, 1000)), more = std::ldexp(1.0, std::max(60 - e - 1000, 0));
+    for (int m = 0; m < M; m++) P[(k * M + m) * TC + c] = fx_limbs(fx_round(src[((size_t)k * M + m) * N + i] * up * more));
+  }
+}
+
+// the P2 reconstruction's tiles (FxTile) of the FP64 form
+int upload_fx_tiles(const ucns_mesh* m, const HostArrays& h, unsigned char** dst) {
+  using T = FxTile;
+  const int nd = m->nd, rec = T::record(nd);
+  const int64_t N = m->N, tiles = (N + T::TC - 1) / T::TC;
+  std::vector<unsigned char> b((size_t)tiles * rec, 0);
+#pragma omp parallel for schedule(static)
+  for (int64_t t = 0; t < tiles; t++) {
+    unsigned char* r = b.data() + (size_t)t * rec;
+    for (int c = 0; c < T::TC && t * T::TC + c < N; c++) {
+      const int64_t i = t * T::TC + c;
+      int32_t* id = reinterpret_cast<int32_t*>(r + T::C_ID);
+      for (int mm = 0; mm < T::MC; mm++) id[mm * T::TC + c] = h.sc[(size_t)mm * N + i];
+      fixed_rows(h.Pc.data(), T::K, T::MC, N, i, T::TC, c, reinterpret_cast<int2*>(r),
+                 reinterpret_cast<int16_t*>(r + T::C_EXP));
+      if (nd == 0) continue;
+      unsigned char* d = r + T::CENTRAL;
+      id = reinterpret_cast<int32_t*>(d + T::d_id(nd));
+      for (int mm = 0; mm < nd * T::MD; mm++) id[mm * T::TC + c] = h.sd[(size_t)mm * N + i];
+      fixed_rows(h.Pd.data(), nd * 3, T::MD, N, i, T::TC, c, reinterpret_cast<int2*>(d),
+                 reinterpret_cast<int16_t*>(d + T::d_exp(nd)));
+    }
+  }
+  return upload(dst, b);
+}
+
 template <typename T>
 int alloc(T** dst, size_t n) {
   if (cudaMalloc((void**)dst, n * sizeof(T)) != cudaSuccess)
@@ -387,6 +426,16 @@ int launch_face_ho(ucns_mesh* m, cudaStream_t s) {
   return UCNS_OK;
 }
 
+// P2, FP64 form
+template <bool WENO, int ND, bool GATED, bool WALLS = false>
+int launch_fx_tiles(const ReconArgs& a, cudaStream_t s) {
+  using T = FxTile;
+  UCNS_CUDA(cudaFuncSetAttribute(k_recon<WENO, ND, GATED, WALLS>, cudaFuncAttributeMaxDynamicSharedMemorySize, T::SMEM));
+  k_recon<WENO, ND, GATED, WALLS><<<(unsigned)((a.N + T::TC - 1) / T::TC), T::THREADS, T::SMEM, s>>>(a);
+  UCNS_CUDA(cudaGetLastError());
+  return UCNS_OK;
+}
+
 int launch_recon_raw(ucns_mesh* m, const double* U, cudaStream_t s) {
   if (mixed(m)) return launch_recon_mx(m, U, s);
   if (m->K > 9) return launch_recon_ho(m, U, s);
@@ -394,8 +443,9 @@ int launch_recon_raw(ucns_mesh* m, const double* U, cudaStream_t s) {
   a.U = U;
   a.sc = m->d.sc;
   a.Pc = m->d.Pc;
-  a.sd = m->d.sd;
-  a.Pd = m->d.Pd;
+  a.tiles = m->d.fxt;
+  a.nd = m->nd;
+  a.err = m->d.err;
   a.mom = m->d.mom;
   a.inv_h = m->d.inv_h;
   a.coef = m->d.coef;
@@ -408,31 +458,20 @@ int launch_recon_raw(ucns_mesh* m, const double* U, cudaStream_t s) {
   a.lams = 1.0 / lsum;
   a.lamc = m->P.lambda_central;
   a.eps = m->P.epsilon;
-  const unsigned g = nblocks((size_t)m->N * 5, kFlatThreads);
   const bool gated = a.gate != nullptr;
   const bool walls = m->n_boundary > 0;
-  if (m->K == 3)
-    k_recon<1, false, 6, false><<<g, kFlatThreads, 0, s>>>(a);
-  else if (m->nd == 0)
-    k_recon<2, false, 6, false><<<g, kFlatThreads, 0, s>>>(a);
-  else if (walls && m->nd == 6)
-    k_recon<2, true, 6, false, true><<<g, kFlatThreads, 0, s>>>(a);
-  else if (walls && m->nd == 5)
-    k_recon<2, true, 5, false, true><<<g, kFlatThreads, 0, s>>>(a);
-  else if (walls)
-    k_recon<2, true, 4, false, true><<<g, kFlatThreads, 0, s>>>(a);
-  else if (m->nd == 5)
-    k_recon<2, true, 5, false><<<g, kFlatThreads, 0, s>>>(a);
-  else if (m->nd == 6 && gated)
-    k_recon<2, true, 6, true><<<g, kFlatThreads, 0, s>>>(a);
-  else if (m->nd == 6)
-    k_recon<2, true, 6, false><<<g, kFlatThreads, 0, s>>>(a);
-  else if (gated)
-    k_recon<2, true, 4, true><<<g, kFlatThreads, 0, s>>>(a);
-  else
-    k_recon<2, true, 4, false><<<g, kFlatThreads, 0, s>>>(a);
-  UCNS_CUDA(cudaGetLastError());
-  return UCNS_OK;
+  if (m->K == 3) {
+    k_recon_p1<<<nblocks((size_t)m->N * 5, kFlatThreads), kFlatThreads, 0, s>>>(a);
+    UCNS_CUDA(cudaGetLastError());
+    return UCNS_OK;
+  }
+  if (m->nd == 0) return launch_fx_tiles<false, 6, false>(a, s);
+  if (walls && m->nd == 6) return launch_fx_tiles<true, 6, false, true>(a, s);
+  if (walls && m->nd == 5) return launch_fx_tiles<true, 5, false, true>(a, s);
+  if (walls) return launch_fx_tiles<true, 4, false, true>(a, s);
+  if (m->nd == 5) return launch_fx_tiles<true, 5, false>(a, s);
+  if (m->nd == 6) return gated ? launch_fx_tiles<true, 6, true>(a, s) : launch_fx_tiles<true, 6, false>(a, s);
+  return gated ? launch_fx_tiles<true, 4, true>(a, s) : launch_fx_tiles<true, 4, false>(a, s);
 }
 
 int launch_face_raw(ucns_mesh* m, cudaStream_t s) {
@@ -645,8 +684,10 @@ int launch_features(ucns_mesh* m, const double* U, void* X, float* Xf, cudaStrea
   FeatArgs a;
   a.U = U;
   a.Uhl = m->d.Uhl;
-  a.sc = mixed(m) ? m->d.scb : m->d.sc;
-  a.Pc = mixed(m) ? (const void*)m->d.Pcb : (const void*)m->d.Pc;
+  a.sc = m->d.scb;
+  a.Pc = m->d.Pcb;
+  a.tiles = m->d.fxt;
+  a.nd = m->nd;
   a.mom = m->d.mom;
   a.inv_h = m->d.inv_h;
   a.cell = m->d.cellb;
@@ -869,7 +910,7 @@ void device_free(ucns_mesh* m) {
   m->gate_eval_active = false;
   m->gate_fixed = false;
   DeviceMesh& d = m->d;
-  void* ptrs[] = {d.fslot, d.bcell, d.bcount, d.inv_vol, d.vol, d.inv_h, d.dtlen, d.mom, d.sc, d.Pc, d.sd, d.Pd, d.Msi, d.psib, d.hot, d.Msif, d.psibf, d.Pcb, d.Pdb, d.scb, d.sdb, d.cellb, d.sda, d.Pda,
+  void* ptrs[] = {d.fslot, d.bcell, d.bcount, d.inv_vol, d.vol, d.inv_h, d.dtlen, d.mom, d.sc, d.Pc, d.sd, d.Pd, d.fxt, d.Msi, d.psib, d.hot, d.Msif, d.psibf, d.Pcb, d.Pdb, d.scb, d.sdb, d.cellb, d.sda, d.Pda,
                   d.inv_hf, d.fpenf, d.cf, d.fo, d.fn, d.dvalid, d.fq, d.fqf, d.fpen, d.coef, d.coeff, d.Uhl, d.G,
                   d.Ustage, d.Uacc, d.Uhost, d.red, d.dt, d.err, d.dt_part, d.dt_count};
   for (void* p : ptrs)
@@ -1054,9 +1095,11 @@ static int device_upload(ucns_mesh* m, const ucns_params* p, const HostArrays& h
     for (int j = 0; j < m->nfc; j++) cf[(size_t)j * m->N + i] = m->cf[(size_t)i * m->nfc + j];
   for (int64_t f = 0; f < m->F; f++)
     if (fn[f] < 0) fn[f] = -1 - (int32_t)h.fkind[f];  // a boundary face carries its kind
+  // at P2 and in the mixed form the stencil ids lie in the reconstruction's tiles
+  const bool tiled = m->K == 9 || p->precision == UCNS_PREC_MIXED;
   if ((rc = upload(&d.vol, h.vol)) || (rc = upload(&d.inv_vol, h.inv_vol)) ||
       (rc = upload(&d.inv_h, h.inv_h)) || (rc = upload(&d.dtlen, h.dtlen)) ||
-      (rc = upload(&d.mom, h.mom)) || (rc = upload(&d.sc, h.sc)) || (rc = upload(&d.sd, h.sd)) ||
+      (rc = upload(&d.mom, h.mom)) || (!tiled && ((rc = upload(&d.sc, h.sc)) || (rc = upload(&d.sd, h.sd)))) ||
       (rc = upload(&d.cf, cf)) || (rc = upload(&d.fo, fo)) || (rc = upload(&d.fn, fn)) ||
       (m->n_boundary > 0 && (rc = upload(&d.dvalid, h.dvalid)))) {
     device_free(m);
@@ -1102,7 +1145,8 @@ static int device_upload(ucns_mesh* m, const ucns_params* p, const HostArrays& h
       device_free(m);
       return rc;
     }
-  } else if ((rc = upload(&d.Pc, h.Pc)) || (rc = upload(&d.Pd, h.Pd)) || (rc = upload(&d.fq, h.fq)) ||
+  } else if ((m->K == 9 && (rc = upload_fx_tiles(m, h, &d.fxt))) ||
+             (m->K != 9 && ((rc = upload(&d.Pc, h.Pc)) || (rc = upload(&d.Pd, h.Pd)))) || (rc = upload(&d.fq, h.fq)) ||
              (rc = upload(&d.fpen, h.fpen)) || (rc = upload(&d.Msi, h.Msi)) || (rc = upload(&d.psib, h.psib)) ||
              (rc = alloc(&d.coef, (size_t)m->NC * m->N * 5))) {
     device_free(m);

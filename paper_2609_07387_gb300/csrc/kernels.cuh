@@ -15,6 +15,9 @@
 
 #include <cstdint>
 
+#include "bulk.cuh"
+#include "fixed.cuh"
+
 namespace ucns {
 
 struct FluxConst {
@@ -23,20 +26,41 @@ struct FluxConst {
 
 struct ReconArgs {
   const double* __restrict__ U;  // [5][N]
-  const int32_t* __restrict__ sc;
-  const double* __restrict__ Pc;
-  const int32_t* __restrict__ sd;
-  const double* __restrict__ Pd;
+  const int32_t* __restrict__ sc;  // [6][N] (P1)
+  const double* __restrict__ Pc;   // [3][6][N] (P1)
+  const unsigned char* __restrict__ tiles;  // per 32-cell tile its stencils and least-squares rows (P2, FxTile)
   const double* __restrict__ mom;  // [6][N]
   const double* __restrict__ inv_h;  // [N]
   double* __restrict__ coef;       // [NC][N][5] physical-unit monomial coefficients
   const uint8_t* __restrict__ gate;  // [N]: 0 -> linear weights (null: every cell CWENOZ)
   float* __restrict__ dev;           // [N]: max |omega - lambda| (null: not wanted)
   const uint8_t* __restrict__ dvalid;  // [N] bit s: directional candidate s exists (WALLS kernels)
+  int* err;  // bit 1: a copy wait gave up
   int N;
   double lam0, lams, eps;  // normalised linear weights, epsilon
   double lamc;             // the central stencil's linear weight before normalisation (WALLS kernels)
+  int nd;                  // directional candidates in the records
 };
+
+// The P2 reconstruction's data in the FP64 form, one contiguous record per tile
+// of 32 cells (zero past N): the central rows [9][18][32] as fixed-point limb
+// pairs, the stencil [18][32] and the rows' exponents [9][32], then (CWENOZ) the
+// same of the directional candidates, [nd][3][6][32], [nd][6][32], [nd][3][32].
+struct FxTile {
+  static constexpr int TC = 32, K = 9, MC = 18, MD = 6;
+  static constexpr int THREADS = 5 * TC;
+  static constexpr int C_ID = K * MC * TC * 8, C_EXP = C_ID + MC * TC * 4, CENTRAL = C_EXP + K * TC * 2;
+  __host__ __device__ static constexpr int d_id(int nd) { return nd * 3 * MD * TC * 8; }
+  __host__ __device__ static constexpr int d_exp(int nd) { return d_id(nd) + nd * MD * TC * 4; }
+  __host__ __device__ static constexpr int directional(int nd) { return d_exp(nd) + nd * 3 * TC * 2; }
+  __host__ __device__ static constexpr int record(int nd) { return CENTRAL + directional(nd); }
+  // shared memory: one buffer for the central part, then the directional one, and a barrier for each
+  static constexpr int SMEM = CENTRAL + 16;
+};
+
+static_assert(FxTile::CENTRAL % 16 == 0 && FxTile::directional(4) % 16 == 0 && FxTile::directional(5) % 16 == 0 &&
+                  FxTile::directional(6) % 16 == 0 && FxTile::directional(6) <= FxTile::CENTRAL,
+              "16-byte copies into one buffer");
 
 struct FaceArgs {
   const double* __restrict__ coef;
@@ -165,39 +189,122 @@ __device__ __forceinline__ void viscous_flux(const double U[5], const double g[5
 }
 
 // ------------------------------------------------------- reconstruction
-// thread = (cell i, variable v); tid = 5 i + v
-template <int ORDER, bool WENO, int ND, bool GATED, bool WALLS = false>
-__global__ void __launch_bounds__(256) k_recon(ReconArgs a) {
-  constexpr int K = ORDER == 1 ? 3 : 9;
-  constexpr int MC = 2 * K;
-  constexpr int MD = 6;
+// out[k] = sum over the stencil's members j = ids[m TC], m < M, of the row
+// entries P[(k M + m) TC] (fixed point, row exponents E[k TC]) times U_j - U_i, all
+// in integers (fixed.cuh); ids, P and E in shared memory
+template <int K, int M, int TC>
+__device__ __forceinline__ void fx_contract(const double* __restrict__ Uv, double ui, const int32_t* ids,
+                                            const int2* P, const int16_t* E, double (&out)[K]) {
+  constexpr int B = fx_bits_of(M);
+  double u[M];
+#pragma unroll
+  for (int m = 0; m < M; m++) u[m] = Uv[ids[m * TC]];
+  int2 q[M];
+  int e;
+  fx_differences<M>(u, ui, q, e);
+#pragma unroll
+  for (int k = 0; k < K; k++) {
+    FxAcc acc;
+#pragma unroll
+    for (int m = 0; m < M; m++) fx_mac(acc, P[(k * M + m) * TC], q[m]);
+    out[k] = fx_double(fx_sum(acc), (int)E[k * TC] + e - 2 - B);
+  }
+}
+
+// P1: thread = (cell i, variable v), tid = 5 i + v
+__global__ void __launch_bounds__(256) k_recon_p1(ReconArgs a) {
   const int tid = blockIdx.x * blockDim.x + threadIdx.x;
   const int i = tid / 5, v = tid - 5 * (tid / 5);
   if (i >= a.N) return;
   const int N = a.N;
   const double* __restrict__ Uv = a.U + (size_t)v * N;
   const double ui = Uv[i];
+  double ao[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+  for (int m = 0; m < 6; m++) {
+    const double d = Uv[__ldg(&a.sc[(size_t)m * N + i])] - ui;
+#pragma unroll
+    for (int k = 0; k < 3; k++) ao[k] = fma(__ldg(&a.Pc[((size_t)k * 6 + m) * N + i]), d, ao[k]);
+  }
+  const double ih = __ldg(&a.inv_h[i]);
+  double* out = a.coef + (size_t)i * 5 + v;
+  const size_t st = (size_t)N * 5;
+  out[0] = ui;
+#pragma unroll
+  for (int k = 0; k < 3; k++) out[(k + 1) * st] = ao[k] * ih;
+}
+
+// P2: one block per 32-cell tile, thread = (cell c, variable v) = 5 c + v.  One
+// thread brings the tile's central part into shared memory by a bulk copy, and the
+// directional part into the same buffer once the central contraction is done; the
+// waits are bounded.  Bound by the FP64 pipe and, at four blocks of five warps per
+// SM, by its latency: with FP64 contractions, streamed from global memory by one
+// thread per (cell, variable), the kernel took 2435 us at 72 x 80 x 88 with 73 % of
+// the pipe's FMA rate.  Contractions in integers from global memory 1970 us (the
+// loads' latency at 12 warps per SM), from shared memory tiles 1648, with the
+// differences in integers too and one division for all weights 1192 (3, 4, 5
+// blocks per SM: 1210, 1192, 1229).
+template <bool WENO, int ND, bool GATED, bool WALLS = false>
+__global__ void __launch_bounds__(FxTile::THREADS, 4) k_recon(ReconArgs a) {
+  using T = FxTile;
+  constexpr int K = T::K, TC = T::TC;
+  extern __shared__ __align__(128) unsigned char smem[];
+  uint64_t* bar = reinterpret_cast<uint64_t*>(smem + T::CENTRAL);
+  const int t = threadIdx.x, tile = blockIdx.x;
+  const int c = t / 5, v = t - 5 * (t / 5);
+  const unsigned char* rec = a.tiles + (size_t)tile * T::record(WENO ? ND : a.nd);
+  if (t == 0) {
+    bar_init(&bar[0]);
+    bar_init(&bar[1]);
+  }
+  __syncthreads();
+  if (t == 0) {
+    bar_expect(&bar[0], T::CENTRAL);
+    bulk_load(smem, rec, T::CENTRAL, &bar[0]);
+  }
+  const int N = a.N;
+  const bool live = tile * TC + c < N;
+  const int i = live ? tile * TC + c : N - 1;
+  const double* __restrict__ Uv = a.U + (size_t)v * N;
+  const double ui = Uv[i];
+  const bool ok = bar_wait(&bar[0], 0);
+  if (__syncthreads_or(!ok)) {
+    if (t == 0) atomicOr(a.err, 2);
+    bar_wait(&bar[0], 0);  // the copy into this block's shared memory ends before it exits
+    return;
+  }
   double ao[K];
-#pragma unroll
-  for (int k = 0; k < K; k++) ao[k] = 0.0;
-#pragma unroll 6
-  for (int m = 0; m < MC; m++) {
-    const int j = __ldg(&a.sc[(size_t)m * N + i]);
-    const double d = Uv[j] - ui;
-#pragma unroll
-    for (int k = 0; k < K; k++) ao[k] = fma(__ldg(&a.Pc[((size_t)k * MC + m) * N + i]), d, ao[k]);
-  }
-  double c[K];
+  fx_contract<K, T::MC, TC>(Uv, ui, reinterpret_cast<const int32_t*>(smem + T::C_ID) + c,
+                            reinterpret_cast<const int2*>(smem) + c, reinterpret_cast<const int16_t*>(smem + T::C_EXP) + c,
+                            ao);
+  double cf[K];
   double S[6];
-  if (ORDER == 2) {
 #pragma unroll
-    for (int q = 0; q < 6; q++) S[q] = __ldg(&a.mom[(size_t)q * N + i]);
-  }
+  for (int q = 0; q < 6; q++) S[q] = __ldg(&a.mom[(size_t)q * N + i]);
   bool weno = WENO;
   if (GATED) weno = weno && a.gate[i];
+  // every read of the central part is done; whether any cell of the tile needs the directional one
+  if constexpr (WENO) {
+    bool any = true;
+    if (GATED) any = __syncthreads_or(weno);
+    else __syncthreads();
+    if (any) {
+      if (t == 0) {
+        bar_expect(&bar[1], T::directional(ND));
+        bulk_load(smem, rec + T::CENTRAL, T::directional(ND), &bar[1]);
+      }
+      const bool okd = bar_wait(&bar[1], 0);
+      if (__syncthreads_or(!okd)) {
+        if (t == 0) atomicOr(a.err, 2);
+        bar_wait(&bar[1], 0);
+        return;
+      }
+    }
+  }
+  if (!live) return;
   if (!weno) {
 #pragma unroll
-    for (int k = 0; k < K; k++) c[k] = ao[k];
+    for (int k = 0; k < K; k++) cf[k] = ao[k];
   } else {
     // WALLS: a cell on a boundary has no directional candidate across it;
     // the linear weights are normalised over the candidates it has
@@ -207,34 +314,30 @@ __global__ void __launch_bounds__(256) k_recon(ReconArgs a) {
     for (int s = 0; s < ND; s++) {
       b[s][0] = b[s][1] = b[s][2] = 0.0;
       if (WALLS && !((valid >> s) & 1u)) continue;
-#pragma unroll
-      for (int r = 0; r < MD; r++) {
-        const int j = __ldg(&a.sd[((size_t)s * MD + r) * N + i]);
-        const double d = Uv[j] - ui;
-#pragma unroll
-        for (int k = 0; k < 3; k++)
-          b[s][k] = fma(__ldg(&a.Pd[(((size_t)s * 3 + k) * MD + r) * N + i]), d, b[s][k]);
-      }
+      fx_contract<3, T::MD, TC>(Uv, ui, reinterpret_cast<const int32_t*>(smem + T::d_id(ND)) + s * T::MD * TC + c,
+                                reinterpret_cast<const int2*>(smem) + s * 3 * T::MD * TC + c,
+                                reinterpret_cast<const int16_t*>(smem + T::d_exp(ND)) + s * 3 * TC + c, b[s]);
     }
-    // smoothness indicators in xi units (h = V^(1/3)):
+    // smoothness indicators in xi units (h = V^(1/3)), H the Hessian of p_opt:
     //   SI = (1/V) int |grad_xi p|^2 + sum_{|beta|=2} (d^beta_xi p)^2
-    const double qx0 = 2.0 * ao[3], qx1 = ao[6], qx2 = ao[7];
-    const double qy0 = ao[6], qy1 = 2.0 * ao[4], qy2 = ao[8];
-    const double qz0 = ao[7], qz1 = ao[8], qz2 = 2.0 * ao[5];
-    auto quad = [&](double x0, double x1, double x2) {
-      return S[0] * x0 * x0 + S[1] * x1 * x1 + S[2] * x2 * x2 +
-             2.0 * (S[3] * x0 * x1 + S[4] * x0 * x2 + S[5] * x1 * x2);
-    };
-    const double SI0 = ao[0] * ao[0] + ao[1] * ao[1] + ao[2] * ao[2] + quad(qx0, qx1, qx2) +
-                       quad(qy0, qy1, qy2) + quad(qz0, qz1, qz2) +
-                       4.0 * (ao[3] * ao[3] + ao[4] * ao[4] + ao[5] * ao[5]) + ao[6] * ao[6] +
-                       ao[7] * ao[7] + ao[8] * ao[8];
-    double SI[ND];
-    double tau = 0.0;
+    //      = |a|^2 + tr(S H^2) + H_xx^2 + H_yy^2 + H_zz^2 + H_xy^2 + H_xz^2 + H_yz^2
+    const double hx = 2.0 * ao[3], hy = 2.0 * ao[4], hz = 2.0 * ao[5], xy = ao[6], xz = ao[7], yz = ao[8];
+    const double oxy = xy * xy, oxz = xz * xz, oyz = yz * yz;
+    const double bx = fma(hx, hx, oxy + oxz), by = fma(hy, hy, oxy + oyz), bz = fma(hz, hz, oxz + oyz);
+    const double bxy = fma(xy, hx + hy, xz * yz), bxz = fma(xz, hx + hz, xy * yz), byz = fma(yz, hy + hz, xy * xz);
+    double SI0 = fma(ao[0], ao[0], fma(ao[1], ao[1], ao[2] * ao[2]));
+    SI0 = fma(S[0], bx, fma(S[1], by, fma(S[2], bz, SI0)));
+    SI0 = fma(2.0, fma(S[3], bxy, fma(S[4], bxz, S[5] * byz)), SI0);
+    SI0 += fma(hx, hx, fma(hy, hy, fma(hz, hz, oxy + oxz + oyz)));
+    // tau and the denominators D = eps + SI (an absent candidate takes 1 and no part)
+    double D[ND + 1], tau = 0.0;
+    D[0] = a.eps + SI0;
 #pragma unroll
     for (int s = 0; s < ND; s++) {
-      SI[s] = b[s][0] * b[s][0] + b[s][1] * b[s][1] + b[s][2] * b[s][2];
-      if (!WALLS || ((valid >> s) & 1u)) tau += fabs(SI0 - SI[s]);
+      const double si = fma(b[s][0], b[s][0], fma(b[s][1], b[s][1], b[s][2] * b[s][2]));
+      const bool on = !WALLS || ((valid >> s) & 1u);
+      if (on) tau += fabs(SI0 - si);
+      D[s + 1] = on ? a.eps + si : 1.0;
     }
     double lam0 = a.lam0, lams = a.lams;
     if (WALLS) {
@@ -245,47 +348,77 @@ __global__ void __launch_bounds__(256) k_recon(ReconArgs a) {
     } else {
       tau *= (1.0 / ND);
     }
-    // omega~_s = lambda_s (1 + tau / (eps + SI_s)), normalised
-    const double w0 = lam0 * (1.0 + tau / (a.eps + SI0));
-    double ws[ND];
-    double wsum = w0;
+    // omega~_s = lambda_s (1 + x_s), x_s = tau / D_s, normalised by their sum 1 + lambda_0
+    // x_0 + lambda sum x_s (the lambdas add up to 1).  The combination p = omega_0 p_1 +
+    // sum omega_s p_s with p_1 = (p_opt - sum lambda_s p_s)/lambda_0 is r0 p_opt + sum e_s
+    // p_s, r0 = (1 + x_0)/sum, e_s = lambda (x_s - x_0)/sum.  Over the common
+    // denominator of all x (Q_s = the product of the other D) that takes one division.
+    double r0, es[ND];
+    int small = 0x7fffffff, large = 0;
 #pragma unroll
-    for (int s = 0; s < ND; s++) {
-      ws[s] = (!WALLS || ((valid >> s) & 1u)) ? lams * (1.0 + tau / (a.eps + SI[s])) : 0.0;
-      wsum += ws[s];
+    for (int s = 0; s <= ND; s++) {
+      const int hi = __double2hiint(D[s]);
+      small = min(small, hi);
+      large = max(large, hi);
     }
-    const double iws = 1.0 / wsum;
-    if (a.dev) {  // deviation of the nonlinear from the linear weights (training labels)
-      double dv = fabs(w0 * iws - lam0);
+    if (small >= (1023 - 140) << 20 && large <= (1023 + 140) << 20) {  // seven factors in [2^-140, 2^141]: no overflow
+      double pre[ND + 1], Q[ND + 1], post = 1.0;
+      pre[0] = 1.0;
 #pragma unroll
-      for (int s = 0; s < ND; s++) dv = fmax(dv, fabs(ws[s] * iws - lams));
+      for (int s = 0; s < ND; s++) pre[s + 1] = s == 0 ? D[0] : pre[s] * D[s];
+      const double all = pre[ND] * D[ND];
+      double sum = 0.0;
+#pragma unroll
+      for (int s = ND; s >= 0; s--) {
+        Q[s] = s == ND ? pre[s] : (s == 0 ? post : pre[s] * post);
+        post = s == ND ? D[s] : post * D[s];
+        if (s > 0 && (!WALLS || ((valid >> (s - 1)) & 1u))) sum += Q[s];
+      }
+      const double top = fma(tau, Q[0], all);
+      const double iw = 1.0 / fma(tau, fma(lam0, Q[0], lams * sum), all);
+      r0 = top * iw;
+      const double te = tau * lams * iw;
+#pragma unroll
+      for (int s = 0; s < ND; s++) es[s] = te * (Q[s + 1] - Q[0]);
+    } else {
+      const double x0 = tau / D[0];
+      double sum = 0.0;
+#pragma unroll
+      for (int s = 0; s < ND; s++) {
+        es[s] = tau / D[s + 1];
+        if (!WALLS || ((valid >> s) & 1u)) sum += es[s];
+      }
+      const double iw = 1.0 / fma(lam0, x0, fma(lams, sum, 1.0));
+      r0 = (1.0 + x0) * iw;
+#pragma unroll
+      for (int s = 0; s < ND; s++) es[s] = lams * iw * (es[s] - x0);
+    }
+    if (a.dev) {  // deviation of the nonlinear from the linear weights (training labels): lambda_0 (r0 - 1), e_s + lambda (r0 - 1)
+      double dv = fabs(lam0 * (r0 - 1.0));
+#pragma unroll
+      for (int s = 0; s < ND; s++) dv = fmax(dv, fabs(fma(lams, r0 - 1.0, es[s])));
       atomicMax(reinterpret_cast<unsigned int*>(a.dev) + i, __float_as_uint((float)dv));
     }
-    // p = omega_0 p_1 + sum_s omega_s p_s with p_1 = (p_opt - sum lambda_s p_s)/lambda_0
-    const double r0 = (w0 * iws) / lam0;
 #pragma unroll
-    for (int k = 0; k < K; k++) c[k] = r0 * ao[k];
+    for (int k = 0; k < K; k++) cf[k] = r0 * ao[k];
 #pragma unroll
     for (int s = 0; s < ND; s++) {
       if (WALLS && !((valid >> s) & 1u)) continue;
-      const double e = ws[s] * iws - r0 * lams;
 #pragma unroll
-      for (int k = 0; k < 3; k++) c[k] = fma(e, b[s][k], c[k]);
+      for (int k = 0; k < 3; k++) cf[k] = fma(es[s], b[s][k], cf[k]);
     }
   }
   // monomial form: p = c0 + sum_k c_k psi_k(xi), c0 = U_i - sum_{k>=3} c_k mean(psi_k);
   // stored in physical units (psi_k of x - x_i): linear terms / h, quadratic / h^2
   double c0 = ui;
-  if (ORDER == 2) {
 #pragma unroll
-    for (int q = 0; q < 6; q++) c0 = fma(-c[3 + q], S[q], c0);
-  }
+  for (int q = 0; q < 6; q++) c0 = fma(-cf[3 + q], S[q], c0);
   const double ih = __ldg(&a.inv_h[i]), ih2 = ih * ih;
   double* out = a.coef + (size_t)i * 5 + v;
   const size_t st = (size_t)N * 5;
   out[0] = c0;
 #pragma unroll
-  for (int k = 0; k < K; k++) out[(k + 1) * st] = c[k] * (k < 3 ? ih : ih2);
+  for (int k = 0; k < K; k++) out[(k + 1) * st] = cf[k] * (k < 3 ? ih : ih2);
 }
 
 // ----------------------------------------------------------- face flux

@@ -13,14 +13,16 @@ namespace ucns {
 struct FeatArgs {
   const double* __restrict__ U;    // [5][N] (FP64 form)
   const float* __restrict__ Uhl;   // [N][5][2] float pairs of U (mixed form)
-  const int32_t* __restrict__ sc;  // [18][N] (FP64 form) or pair-blocked (mixed form)
-  const void* __restrict__ Pc;     // [9][18][N] double (FP64 form) or pair-blocked float (mixed form)
+  const int32_t* __restrict__ sc;  // pair-blocked (mixed form)
+  const float* __restrict__ Pc;    // pair-blocked (mixed form)
+  const unsigned char* __restrict__ tiles;  // fixed-point rows (FP64 form, FxTile)
   const double* __restrict__ mom;    // [6][N] (FP64 form)
   const double* __restrict__ inv_h;  // [N] (FP64 form)
   const float* __restrict__ cell;    // blocked [tiles][kCellRows][kTC] (mixed form)
   __nv_bfloat16* __restrict__ X;  // [N][32]
   float* __restrict__ Xf;         // [N][32] or null
   int N;
+  int nd;  // directional candidates in the tiles
   float gam;
 };
 
@@ -72,13 +74,16 @@ __device__ __forceinline__ void features_finish(float F[32], const float (&ao)[5
   }
 }
 
-// FP64 form: differences of the FP64 state, FP64 pseudo-inverse rows
+// FP64 form: differences of the FP64 state, fixed-point pseudo-inverse rows rounded to FP32
 __global__ void __launch_bounds__(128) k_features(FeatArgs a) {
   constexpr int K = 9, MC = 18;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= a.N) return;
   const size_t N = a.N;
-  const double* __restrict__ Pc = reinterpret_cast<const double*>(a.Pc);
+  const unsigned char* rec = a.tiles + (size_t)(i / FxTile::TC) * FxTile::record(a.nd);
+  const int2* __restrict__ P = reinterpret_cast<const int2*>(rec) + i % FxTile::TC;
+  const int32_t* __restrict__ ids = reinterpret_cast<const int32_t*>(rec + FxTile::C_ID) + i % FxTile::TC;
+  const int16_t* __restrict__ E = reinterpret_cast<const int16_t*>(rec + FxTile::C_EXP) + i % FxTile::TC;
   const double g = a.gam;
   double Ui[5];
 #pragma unroll
@@ -95,7 +100,7 @@ __global__ void __launch_bounds__(128) k_features(FeatArgs a) {
     for (int k = 0; k < K; k++) ao[v][k] = 0.f;
 #pragma unroll 2
   for (int m = 0; m < MC; m++) {
-    const int j = __ldg(&a.sc[(size_t)m * N + i]);
+    const int j = __ldg(&ids[m * FxTile::TC]);
     double Uj[5];
     float d[5];
 #pragma unroll
@@ -110,10 +115,18 @@ __global__ void __launch_bounds__(128) k_features(FeatArgs a) {
     }
 #pragma unroll
     for (int k = 0; k < K; k++) {
-      const float P = (float)Pc[((size_t)k * MC + m) * N + i];
+      const int2 q = __ldg(&P[(k * MC + m) * FxTile::TC]);
+      // 2^60 P_km 2^-E_k, rounded once; the row's scale follows after the sum
+      const float p = __ll2float_rn(((long long)q.x << 30) + q.y);
 #pragma unroll
-      for (int v = 0; v < 5; v++) ao[v][k] = fmaf(P, d[v], ao[v][k]);
+      for (int v = 0; v < 5; v++) ao[v][k] = fmaf(p, d[v], ao[v][k]);
     }
+  }
+#pragma unroll
+  for (int k = 0; k < K; k++) {
+    const int e = (int)__ldg(&E[k * FxTile::TC]) - 60;
+#pragma unroll
+    for (int v = 0; v < 5; v++) ao[v][k] = ldexpf(ao[v][k], e);
   }
   float S[6];
 #pragma unroll
@@ -129,7 +142,7 @@ __global__ void __launch_bounds__(128, 4) k_features_mx(FeatArgs a) {
   constexpr int K = 9, MC = 18;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= a.N) return;
-  const float* __restrict__ Pc = reinterpret_cast<const float*>(a.Pc);
+  const float* __restrict__ Pc = a.Pc;
   const float2* __restrict__ hl2 = reinterpret_cast<const float2*>(a.Uhl);  // a row: (hi, lo) of 5 variables
   const float g = a.gam;
   float hi[5], lo[5];

@@ -36,6 +36,7 @@ struct DeviceMesh {
   double* Pc = nullptr;       // [K][Mc][N] central pseudo-inverse
   int32_t* sd = nullptr;      // [nd][Md][N] directional stencils
   double* Pd = nullptr;       // [nd][Kd][Md][N]
+  unsigned char* fxt = nullptr;  // FP64 form at P2: stencils and least-squares rows in fixed point, 32-cell tiles
   double* Msi = nullptr;      // P3/P4: [K(K+1)/2][N] smoothness-indicator matrix (upper triangle, row-major)
   float* hot = nullptr;       // P3/P4 mixed form: stencil ids and FP32 pseudo-inverses in 64-cell tiles; FP32 Msi, psib
   float* Msif = nullptr;

@@ -1,0 +1,75 @@
+"""The FP64 form's fixed-point contractions (csrc/fixed.cuh) where they can go
+wrong: ragged tiles of every element kind, weights whose common denominator
+leaves the product range, states whose differences are subnormal before they
+are aligned, and non-finite states; against the oracle at its FP64 bar (1e-12
+of the summed-term scale, tests/test_gpu_parity.py)."""
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_2609_07387_gb300 import inputs as I
+from paper_2609_07387_gb300 import ucns
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def _mesh(kind, n):
+    nodes, cells, box = I.hex_lattice(n, jitter=0.1, seed=5)
+    if kind == "tets":
+        cells = I.split_tets(cells)
+    if kind == "prisms":
+        cells = I.split_prisms(cells)
+    if kind == "pyramids":
+        nodes, cells = I.split_pyramids(nodes, cells)
+    if kind == "walls":
+        box = np.array([box[0], box[1], 0.0])
+    return nodes, cells, box
+
+
+def _both(kind, n, order, scheme, Re=0.0, eps=1e-6, mach=0.5):
+    nodes, cells, box = _mesh(kind, n)
+    m = ucns.Mesh(nodes, cells, box, ucns.Params(order=order, scheme=scheme, Re=Re, Mach=mach, eps=eps))
+    oc = O.Case(nodes, cells, box, O.Params(order=order, scheme=scheme, Re=Re, Mach=mach, eps=eps))
+    return m, oc, I.noisy_state(nodes, cells, mach, 0.05, seed=6)
+
+
+def _residual(m, U):
+    R = m.residual(torch.from_numpy(np.ascontiguousarray(m.to_internal(U))).cuda())
+    return m.to_user(R.cpu().numpy())
+
+
+# 210, 1050, 420, 1260 and 210 cells: the last 32-cell tile holds 18, 26, 4, 12 and 18;
+# eps 1e-60 with a uniform z momentum and states scaled by 2^200 leave the range in
+# which the weights share one denominator
+@pytest.mark.parametrize("kind,n,order,scheme", [
+    ("hexes", (5, 6, 7), 2, 1), ("hexes", (5, 6, 7), 2, 0), ("tets", (5, 5, 7), 2, 1), ("prisms", (5, 6, 7), 2, 1),
+    ("pyramids", (5, 6, 7), 2, 1), ("walls", (5, 6, 7), 2, 1)])
+@pytest.mark.parametrize("eps,scale", [(1e-6, 0), (1e-60, 0), (1e-6, 200)])
+def test_residual_on_ragged_tiles(kind, n, order, scheme, eps, scale):
+    m, oc, U = _both(kind, n, order, scheme, eps=eps)
+    if eps < 1e-50:
+        U[3] = 0.0
+    U = U * 2.0 ** scale
+    R, (Rc, S) = _residual(m, U), oc.residual_terms(U)
+    err = np.abs(R - Rc).max(axis=1) / np.maximum(S.max(axis=1), 1e-300)
+    print(kind, eps, scale, err)
+    assert np.all(err <= 1e-12)
+
+
+# The Euler residual with linear weights scales with the state; powers of two scale
+# exactly through every operation, also where the state lies below the range in
+# which differences are aligned directly (2^-962)
+@pytest.mark.parametrize("order", [2])
+@pytest.mark.parametrize("k", [-962, 600])
+def test_power_of_two_states_scale_exactly(order, k):
+    m, _, U = _both("hexes", (9, 9, 10), order, 0, mach=1.0)
+    assert np.array_equal(_residual(m, U * 2.0 ** k), _residual(m, U) * 2.0 ** k)
+
+
+@pytest.mark.parametrize("order", [2])
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+def test_non_finite_states_stay_visible(order, bad):
+    m, oc, U = _both("hexes", (11, 11, 12), order, 0)
+    U[1, 700] = bad
+    assert np.array_equal(np.isfinite(_residual(m, U)), np.isfinite(oc.residual(U)))
