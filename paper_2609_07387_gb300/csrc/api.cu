@@ -171,12 +171,12 @@ FluxConst flux_const(const ucns_params& p) {
   FluxConst c;
   c.gam = p.gamma;
   c.gm1 = p.gamma - 1.0;
+  c.half_gm1 = 0.5 * c.gm1;
   const double Rg = 1.0 / (p.gamma * p.mach * p.mach);
   const bool visc = p.reynolds > 0.0;
   c.mu = visc ? 1.0 / p.reynolds : 0.0;
   const double cp = p.gamma * Rg / (p.gamma - 1.0);
-  c.kap = visc ? c.mu * cp / p.prandtl : 0.0;
-  c.gm1_over_R = (p.gamma - 1.0) / Rg;
+  c.k_e = visc ? c.mu * cp / p.prandtl * c.gm1 / Rg : 0.0;
   return c;
 }
 
@@ -185,9 +185,9 @@ FluxConstF flux_const_f(const ucns_params& p) {
   FluxConstF c;
   c.gam = (float)d.gam;
   c.gm1 = (float)d.gm1;
+  c.half_gm1 = (float)d.half_gm1;
   c.mu = (float)d.mu;
-  c.kap = (float)d.kap;
-  c.gm1_over_R = (float)d.gm1_over_R;
+  c.k_e = (float)d.k_e;
   const double p_ref = 1.0 / (p.gamma * p.mach * p.mach);
   c.p_ref = (float)p_ref;
   c.H_ref = (float)(p.gamma * p_ref / (p.gamma - 1.0));

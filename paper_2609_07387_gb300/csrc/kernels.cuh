@@ -21,7 +21,7 @@
 namespace ucns {
 
 struct FluxConst {
-  double gam, gm1, mu, kap, gm1_over_R;  // gm1_over_R = (gamma-1)/R_gas
+  double gam, gm1, half_gm1, mu, k_e;  // k_e = kappa (gamma-1)/R_gas: heat flux per gradient of the inner energy
 };
 
 struct ReconArgs {
@@ -94,13 +94,35 @@ struct RKArgs {
 };
 
 // --------------------------------------------------------------- fluxes
-__device__ __forceinline__ void phys_flux(const double U[5], double ir, const double u[3], double p,
+// The FP64 face kernels are bound by the FP64 pipe, where a division or a square
+// root takes 7.5 and a comparison one of its issue slots: both fluxes are written
+// for the fewest FP64 operations: two divisions less than the difference form of
+// the star flux and Roe's enthalpy, 1/rho once in the viscous flux, the energy
+// gradient by its normal part (k_face<2> at 72 x 80 x 88 5418 -> 4756 us; the mixed
+// form's fluxes, written alike, k_face_mx<2> at 96^3 210 -> 196 us).
+__device__ __forceinline__ void phys_flux(const double U[5], const double u[3], double p,
                                           double un, const double n[3], double F[5]) {
   F[0] = U[0] * un;
   F[1] = U[1] * un + p * n[0];
   F[2] = U[2] * un + p * n[1];
   F[3] = U[3] * un + p * n[2];
   F[4] = (U[4] + p) * un;
+}
+
+// the star-region flux F + S (U* - U) of one side (rho (S - u_n) = m, contact
+// speed Ss), which is the flux of the star state itself: rho* Ss times (1, u + (Ss
+// - u_n) n, E*/rho*) plus p* (0, n, Ss), with p* = p + m (Ss - u_n)
+__device__ __forceinline__ void star_flux(const double U[5], double ir, const double u[3], double p, double un,
+                                          double m, double S, double Ss, const double n[3], double F[5]) {
+  const double r = 1.0 / (S - Ss), ds = Ss - un;
+  const double rho = m * r, ps = fma(m, ds, p);
+  F[0] = rho * Ss;
+  const double cn = fma(F[0], ds, ps);
+#pragma unroll
+  for (int d = 0; d < 3; d++) F[1 + d] = fma(F[0], u[d], cn * n[d]);
+  // rho* (E/rho + (Ss - u_n)(Ss + p/m)), rho*/m = r
+  const double Es = fma(rho, fma(ds, Ss, U[4] * ir), (ds * p) * r);
+  F[4] = Ss * (Es + ps);
 }
 
 // HLLC (Toro, Spruce & Speares) with Einfeldt/Roe wave-speed bounds; flux
@@ -118,74 +140,83 @@ __device__ __forceinline__ void hllc_flux(const double UL[5], const double UR[5]
   const double pR = c.gm1 * (UR[4] - 0.5 * (UR[1] * uR[0] + UR[2] * uR[1] + UR[3] * uR[2]));
   const double unL = uL[0] * n[0] + uL[1] * n[1] + uL[2] * n[2];
   const double unR = uR[0] * n[0] + uR[1] * n[1] + uR[2] * n[2];
-  const double aL = sqrt(c.gam * pL * irL), aR = sqrt(c.gam * pR * irR);
+  const double a2L = c.gam * pL * irL, a2R = c.gam * pR * irR;
+  const double aL = sqrt(a2L), aR = sqrt(a2R);
+  // Roe averages with the weights w = sqrt(rho) / (sqrt(rho_L) + sqrt(rho_R)): u~_n,
+  // and the sound speed of the averaged enthalpy, a~^2 = (gamma-1)(H~ - |u~|^2/2) =
+  // w_L a_L^2 + w_R a_R^2 + (gamma-1)/2 w_L w_R |u_R - u_L|^2
   const double iw = 1.0 / (sL + sR);
-  // Roe averages: sqrt(rho) u = m / sqrt(rho), sqrt(rho) H = (E + p) / sqrt(rho)
-  const double ut0 = (UL[1] * qL + UR[1] * qR) * iw, ut1 = (UL[2] * qL + UR[2] * qR) * iw,
-               ut2 = (UL[3] * qL + UR[3] * qR) * iw;
-  const double Ht = ((UL[4] + pL) * qL + (UR[4] + pR) * qR) * iw;
-  const double at = sqrt(c.gm1 * (Ht - 0.5 * (ut0 * ut0 + ut1 * ut1 + ut2 * ut2)));
-  const double utn = ut0 * n[0] + ut1 * n[1] + ut2 * n[2];
+  const double wL = sL * iw, wR = sR * iw;
+  const double d0 = uR[0] - uL[0], d1 = uR[1] - uL[1], d2 = uR[2] - uL[2];
+  const double at = sqrt(fma(c.half_gm1 * wL * wR, fma(d0, d0, fma(d1, d1, d2 * d2)), fma(wL, a2L, wR * a2R)));
+  const double utn = fma(wL, unL, wR * unR);
   const double SL = fmin(unL - aL, utn - at);
   const double SR = fmax(unR + aR, utn + at);
   const double mL = rL * (SL - unL), mR = rR * (SR - unR);
   const double Ss = (pR - pL + unL * mL - unR * mR) / (mL - mR);
   if (0.0 <= SL) {
-    phys_flux(UL, irL, uL, pL, unL, n, F);
+    phys_flux(UL, uL, pL, unL, n, F);
   } else if (0.0 <= Ss) {
-    phys_flux(UL, irL, uL, pL, unL, n, F);
-    const double f = mL / (SL - Ss), ds = Ss - unL;
-    const double Us4 = f * (UL[4] * irL + ds * (Ss + pL / mL));
-    F[0] += SL * (f - UL[0]);
-    F[1] += SL * (f * (uL[0] + ds * n[0]) - UL[1]);
-    F[2] += SL * (f * (uL[1] + ds * n[1]) - UL[2]);
-    F[3] += SL * (f * (uL[2] + ds * n[2]) - UL[3]);
-    F[4] += SL * (Us4 - UL[4]);
+    star_flux(UL, irL, uL, pL, unL, mL, SL, Ss, n, F);
   } else if (0.0 <= SR) {
-    phys_flux(UR, irR, uR, pR, unR, n, F);
-    const double f = mR / (SR - Ss), ds = Ss - unR;
-    const double Us4 = f * (UR[4] * irR + ds * (Ss + pR / mR));
-    F[0] += SR * (f - UR[0]);
-    F[1] += SR * (f * (uR[0] + ds * n[0]) - UR[1]);
-    F[2] += SR * (f * (uR[1] + ds * n[1]) - UR[2]);
-    F[3] += SR * (f * (uR[2] + ds * n[2]) - UR[3]);
-    F[4] += SR * (Us4 - UR[4]);
+    star_flux(UR, irR, uR, pR, unR, mR, SR, Ss, n, F);
   } else {
-    phys_flux(UR, irR, uR, pR, unR, n, F);
+    phys_flux(UR, uR, pR, unR, n, F);
   }
 }
 
-// Viscous flux F_v . n from the face state and the conserved gradient.
-__device__ __forceinline__ void viscous_flux(const double U[5], const double g[5][3],
+// Viscous flux F_v . n from a face state (up to a common factor with g) and the
+// conserved gradients: g of density and momenta, g4n = grad(rho E) . n.  Written
+// with rho grad u = grad m - u grad rho, so that the one 1/rho enters at the end:
+//   t_a = (mu/rho)(G_aj n_j + G_ja n_j - 2/3 tr(G) n_a),  G = rho grad u
+//   rho grad e . n = grad(rho E) . n - E grad rho . n - u_a G_aj n_j
+__device__ __forceinline__ void viscous_flux(const double U[5], const double g[4][3], double g4n,
                                              const double n[3], const FluxConst& c, double Fv[5]) {
   const double ir = 1.0 / U[0];
   const double u[3] = {U[1] * ir, U[2] * ir, U[3] * ir};
-  double gu[3][3];
-#pragma unroll
-  for (int a = 0; a < 3; a++)
-#pragma unroll
-    for (int j = 0; j < 3; j++) gu[a][j] = (g[1 + a][j] - u[a] * g[0][j]) * ir;
-  const double e = U[4] * ir;
-  double qn = 0.0;
-#pragma unroll
-  for (int j = 0; j < 3; j++) {
-    const double de = (g[4][j] - e * g[0][j]) * ir - (u[0] * gu[0][j] + u[1] * gu[1][j] + u[2] * gu[2][j]);
-    qn += de * n[j];
-  }
-  const double div = gu[0][0] + gu[1][1] + gu[2][2];
-  const double tdiv = (2.0 / 3.0) * c.mu * div;
-  double work = 0.0;
-  Fv[0] = 0.0;
+  double G[3][3], dn[3];
 #pragma unroll
   for (int a = 0; a < 3; a++) {
-    double t = 0.0;
 #pragma unroll
-    for (int j = 0; j < 3; j++) t += c.mu * (gu[a][j] + gu[j][a]) * n[j];
-    t -= tdiv * n[a];
-    Fv[1 + a] = t;
-    work += u[a] * t;
+    for (int j = 0; j < 3; j++) G[a][j] = fma(-u[a], g[0][j], g[1 + a][j]);
+    dn[a] = fma(G[a][0], n[0], fma(G[a][1], n[1], G[a][2] * n[2]));
   }
-  Fv[4] = work + c.kap * c.gm1_over_R * qn;
+  const double tdiv = (2.0 / 3.0) * (G[0][0] + G[1][1] + G[2][2]);
+  const double mr = c.mu * ir;
+  Fv[0] = 0.0;
+#pragma unroll
+  for (int a = 0; a < 3; a++)
+    Fv[1 + a] = mr * fma(G[0][a], n[0], fma(G[1][a], n[1], fma(G[2][a], n[2], fma(-tdiv, n[a], dn[a]))));
+  const double g0n = fma(g[0][0], n[0], fma(g[0][1], n[1], g[0][2] * n[2]));
+  const double en = fma(-u[0], dn[0], fma(-u[1], dn[1], fma(-u[2], dn[2], fma(-(U[4] * ir), g0n, g4n))));
+  Fv[4] = fma(u[0], Fv[1], fma(u[1], Fv[2], fma(u[2], Fv[3], c.k_e * ir * en)));
+}
+
+// The total flux per unit area at a Gauss point from both sides' states and gs =
+// grad U_L + grad U_R: HLLC, less (VISC) the viscous flux of the penalised face
+// gradient.  2 U_f = U_L + U_R and 2 grad U_f = gs + 2 (alpha/L)(U_R - U_L) n:
+// the viscous flux depends on them only through ratios, so the common factor 2
+// cancels; the energy gradient enters through its normal part alone.
+template <bool VISC>
+__device__ __forceinline__ void point_flux(const double UL[5], const double UR[5], const double gs[5][3],
+                                           const double n[3], double pen2, const FluxConst& c, double F[5]) {
+  hllc_flux(UL, UR, n, c, F);
+  if (VISC) {
+    double Uf2[5], gf2[4][3];
+#pragma unroll
+    for (int v = 0; v < 4; v++) {
+      const double jump2 = pen2 * (UR[v] - UL[v]);
+      Uf2[v] = UL[v] + UR[v];
+#pragma unroll
+      for (int j = 0; j < 3; j++) gf2[v][j] = fma(jump2, n[j], gs[v][j]);
+    }
+    Uf2[4] = UL[4] + UR[4];
+    const double g4n = fma(gs[4][0], n[0], fma(gs[4][1], n[1], fma(gs[4][2], n[2], pen2 * (UR[4] - UL[4]))));
+    double Fv[5];
+    viscous_flux(Uf2, gf2, g4n, n, c, Fv);
+#pragma unroll
+    for (int v = 1; v < 5; v++) F[v] -= Fv[v];
+  }
 }
 
 // ------------------------------------------------------- reconstruction
@@ -503,30 +534,10 @@ __global__ void __launch_bounds__(256) k_face(FaceArgs a) {
   eval_side<ORDER, false>(a.coef, a.N, o, xl, yl, zl, UL, gs);
   if (BND && nb < 0) ghost_state(-1 - nb, UL, n, a.uinf, UR);
   else eval_side<ORDER, true>(a.coef, a.N, nb, xr, yr, zr, UR, gs);
-  double Fc[5];
-  hllc_flux(UL, UR, n, a.c, Fc);
   double flux[5];
-  if (VISC && !BND) {
-    // 2 U_f = U_L + U_R and 2 grad U_f = gs + 2 (alpha/L)(U_R - U_L) n: the viscous
-    // flux depends on the face state only through ratios (u = m/rho, e = E/rho,
-    // grad u = (grad m - u grad rho)/rho), so the common factor 2 cancels
-    const double pen2 = 2.0 * a.fpen[fc];
-    double Uf2[5], gf2[5][3];
+  point_flux<VISC && !BND>(UL, UR, gs, n, VISC && !BND ? 2.0 * a.fpen[fc] : 0.0, a.c, flux);
 #pragma unroll
-    for (int v = 0; v < 5; v++) {
-      const double jump2 = pen2 * (UR[v] - UL[v]);
-      Uf2[v] = UL[v] + UR[v];
-#pragma unroll
-      for (int j = 0; j < 3; j++) gf2[v][j] = fma(jump2, n[j], gs[v][j]);
-    }
-    double Fv[5];
-    viscous_flux(Uf2, gf2, n, a.c, Fv);
-#pragma unroll
-    for (int v = 0; v < 5; v++) flux[v] = (Fc[v] - Fv[v]) * area;
-  } else {
-#pragma unroll
-    for (int v = 0; v < 5; v++) flux[v] = Fc[v] * area;
-  }
+  for (int v = 0; v < 5; v++) flux[v] *= area;
 #pragma unroll
   for (int off = 1; off < NQ; off <<= 1)
 #pragma unroll

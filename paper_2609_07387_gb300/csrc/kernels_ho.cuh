@@ -229,28 +229,10 @@ __global__ void __launch_bounds__(128) k_face_ho(FaceArgs a) {
   double UL[5], UR[5], gs[5][3];  // gs = grad U_L + grad U_R
   eval_side_ho<ORDER, false>(a.coef, a.N, o, xl, yl, zl, UL, gs);
   eval_side_ho<ORDER, true>(a.coef, a.N, nb, xr, yr, zr, UR, gs);
-  double Fc[5];
-  hllc_flux(UL, UR, n, a.c, Fc);
   double flux[5];
-  if (VISC) {
-    // as in k_face: twice the face state and the penalised face gradient
-    const double pen2 = 2.0 * a.fpen[fc];
-    double Uf2[5], gf2[5][3];
+  point_flux<VISC>(UL, UR, gs, n, VISC ? 2.0 * a.fpen[fc] : 0.0, a.c, flux);
 #pragma unroll
-    for (int v = 0; v < 5; v++) {
-      const double jump2 = pen2 * (UR[v] - UL[v]);
-      Uf2[v] = UL[v] + UR[v];
-#pragma unroll
-      for (int j = 0; j < 3; j++) gf2[v][j] = fma(jump2, n[j], gs[v][j]);
-    }
-    double Fv[5];
-    viscous_flux(Uf2, gf2, n, a.c, Fv);
-#pragma unroll
-    for (int v = 0; v < 5; v++) flux[v] = (Fc[v] - Fv[v]) * area;
-  } else {
-#pragma unroll
-    for (int v = 0; v < 5; v++) flux[v] = Fc[v] * area;
-  }
+  for (int v = 0; v < 5; v++) flux[v] *= area;
   // the group's first lane sums its NQ points in point order (every lane takes
   // part in the shuffles; lanes outside a group read group 0 and store nothing)
   const int base = (in_group ? grp : 0) * NQ;

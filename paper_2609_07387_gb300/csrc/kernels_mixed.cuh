@@ -25,7 +25,7 @@
 namespace ucns {
 
 struct FluxConstF {
-  float gam, gm1, mu, kap, gm1_over_R;
+  float gam, gm1, half_gm1, mu, k_e;  // k_e = kappa (gamma-1)/R_gas
   float p_ref, H_ref;  // reference pressure and enthalpy E_ref + p_ref
 };
 
@@ -516,87 +516,65 @@ __device__ __forceinline__ void hllc_flux_mx(const float WL[5], const float WR[5
   const float pL = c.p_ref + ppL, pR = c.p_ref + ppR;
   const float unL = uL[0] * n[0] + uL[1] * n[1] + uL[2] * n[2];
   const float unR = uR[0] * n[0] + uR[1] * n[1] + uR[2] * n[2];
-  const float aL = fsqrt(c.gam * pL * irL), aR = fsqrt(c.gam * pR * irR);
+  const float a2L = c.gam * pL * irL, a2R = c.gam * pR * irR;
+  const float aL = fsqrt(a2L), aR = fsqrt(a2R);
   const float sL = fsqrt(rL), sR = fsqrt(rR), iw = fdiv(1.f, sL + sR);
-  const float ut0 = (sL * uL[0] + sR * uR[0]) * iw, ut1 = (sL * uL[1] + sR * uR[1]) * iw,
-              ut2 = (sL * uL[2] + sR * uR[2]) * iw;
-  // total enthalpy H = (E + p)/rho = (H_ref + E' + p')/rho
-  const float Ht = (sL * (c.H_ref + WL[4] + ppL) * irL + sR * (c.H_ref + WR[4] + ppR) * irR) * iw;
-  const float at = fsqrt(c.gm1 * (Ht - 0.5f * (ut0 * ut0 + ut1 * ut1 + ut2 * ut2)));
-  const float utn = ut0 * n[0] + ut1 * n[1] + ut2 * n[2];
+  // Roe averages as in the FP64 form: a~^2 = w_L a_L^2 + w_R a_R^2 + (gamma-1)/2 w_L w_R |u_R - u_L|^2
+  const float wL = sL * iw, wR = sR * iw;
+  const float e0 = uR[0] - uL[0], e1 = uR[1] - uL[1], e2 = uR[2] - uL[2];
+  const float at = fsqrt(fmaf(c.half_gm1 * wL * wR, fmaf(e0, e0, fmaf(e1, e1, e2 * e2)), fmaf(wL, a2L, wR * a2R)));
+  const float utn = fmaf(wL, unL, wR * unR);
   const float SL = fminf(unL - aL, utn - at);
   const float SR = fmaxf(unR + aR, utn + at);
   const float mL = rL * (SL - unL), mR = rR * (SR - unR);
   const float Ss = fdiv(ppR - ppL + unL * mL - unR * mR, mL - mR);
-  // The flux is that of the upwind side (left when S_L >= 0 or S* >= 0),
-  // plus S (U* - U) of that side in the star region (S_L < 0 on the left,
-  // S_R >= 0 on the right).  Written without branches: the side's
-  // quantities are selected first, so a warp whose faces fall on different
-  // sides runs one path.  Physical flux: momentum with p', energy with the
-  // full E + p.  U* - U with r* = (S* - u_n)/(S - S*): d_rho = rho r*,
-  // d_m = r* m + rho* (S* - u_n) n, d_E = r* E + rho* (S* - u_n)(S* + p/(rho (S - u_n))).
+  // The flux is that of the upwind side's star state (left when S_L >= 0 or S* >=
+  // 0), written without branches: the side's quantities are selected first, and
+  // outside the star region (S_L >= 0 on the left, S_R < 0 on the right) the star
+  // speed is taken as the side's own u_n, where the star flux is the physical
+  // flux.  With s the star speed and r* = (s - u_n)/(S - s): rho* = rho (1 + r*);
+  // momentum with p' (the dropped p_ref n integrates to zero), energy s (E* + p*) =
+  // s (E + p)(1 + r*) + s (s - u_n)(rho* s + m), E + p = H_ref + E' + p'.  The large
+  // parts rho s and H_ref s are rounded once, as in a plain flux.
   const bool left = 0.f <= SL || 0.f <= Ss;
-  const float W0 = left ? WL[0] : WR[0], W1 = left ? WL[1] : WR[1], W2 = left ? WL[2] : WR[2];
-  const float W3 = left ? WL[3] : WR[3], W4 = left ? WL[4] : WR[4];
-  (void)W0;
-  const float r = left ? rL : rR, un = left ? unL : unR, pp = left ? ppL : ppR, p = left ? pL : pR;
+  const float r = left ? rL : rR, un = left ? unL : unR, pp = left ? ppL : ppR;
   const float S = left ? SL : SR, m = left ? mL : mR;
+  const float hp = (left ? WL[4] : WR[4]) + pp;
   const bool in_star = left ? SL < 0.f : 0.f <= SR;
-  F[0] = r * un;
-  F[1] = W1 * un + pp * n[0];
-  F[2] = W2 * un + pp * n[1];
-  F[3] = W3 * un + pp * n[2];
-  F[4] = (W4 + pp) * un + c.H_ref * un;
-  const float ds = Ss - un;
-  const float rs = fdiv(ds, S - Ss);
-  const float rho_s = r + r * rs;
-  const float E = (c.H_ref - c.p_ref) + W4;
-  const float t = rho_s * ds;
-  const float d0 = S * (r * rs);
-  const float d1 = S * fmaf(t, n[0], rs * W1);
-  const float d2 = S * fmaf(t, n[1], rs * W2);
-  const float d3 = S * fmaf(t, n[2], rs * W3);
-  const float d4 = S * fmaf(t, Ss + fdiv(p, m), rs * E);
-  // outside the star region these terms may be inf or NaN (S = S*): selected away
-  F[0] += in_star ? d0 : 0.f;
-  F[1] += in_star ? d1 : 0.f;
-  F[2] += in_star ? d2 : 0.f;
-  F[3] += in_star ? d3 : 0.f;
-  F[4] += in_star ? d4 : 0.f;
+  const float s = in_star ? Ss : un;
+  const float ds = s - un;
+  const float rs = in_star ? fdiv(ds, S - s) : 0.f;
+  F[0] = fmaf(r * rs, s, r * s);
+  const float cn = fmaf(F[0], ds, fmaf(m, ds, pp));
+#pragma unroll
+  for (int d = 0; d < 3; d++) F[1 + d] = fmaf(F[0], left ? uL[d] : uR[d], cn * n[d]);
+  F[4] = fmaf(c.H_ref, s, fmaf(hp, s, s * fmaf(rs, c.H_ref + hp, ds * (F[0] + m))));
 }
 
-// viscous flux in FP32 from the reference-relative face state
-__device__ __forceinline__ void viscous_flux_mx(const float W[5], const float g[5][3], const float n[3],
+// viscous flux in FP32 from the reference-relative face state and the gradients g of
+// density and momenta, g4n = grad(rho E) . n: written as in the FP64 form, with G
+// = rho grad u = grad m - u grad rho and the one 1/rho at the end
+__device__ __forceinline__ void viscous_flux_mx(const float W[5], const float g[4][3], float g4n, const float n[3],
                                                 const FluxConstF& c, float Fv[5]) {
-  const float r = 1.f + W[0];
-  const float ir = fdiv(1.f, r);
+  const float ir = fdiv(1.f, 1.f + W[0]);
   const float u[3] = {W[1] * ir, W[2] * ir, W[3] * ir};
-  float gu[3][3];
-#pragma unroll
-  for (int q = 0; q < 3; q++)
-#pragma unroll
-    for (int j = 0; j < 3; j++) gu[q][j] = (g[1 + q][j] - u[q] * g[0][j]) * ir;
-  const float e = ((c.H_ref - c.p_ref) + W[4]) * ir;
-  float qn = 0.f;
-#pragma unroll
-  for (int j = 0; j < 3; j++) {
-    const float de = (g[4][j] - e * g[0][j]) * ir - (u[0] * gu[0][j] + u[1] * gu[1][j] + u[2] * gu[2][j]);
-    qn += de * n[j];
-  }
-  const float div = gu[0][0] + gu[1][1] + gu[2][2];
-  const float tdiv = (2.f / 3.f) * c.mu * div;
-  float work = 0.f;
-  Fv[0] = 0.f;
+  float G[3][3], dn[3];
 #pragma unroll
   for (int q = 0; q < 3; q++) {
-    float t = 0.f;
 #pragma unroll
-    for (int j = 0; j < 3; j++) t += c.mu * (gu[q][j] + gu[j][q]) * n[j];
-    t -= tdiv * n[q];
-    Fv[1 + q] = t;
-    work += u[q] * t;
+    for (int j = 0; j < 3; j++) G[q][j] = fmaf(-u[q], g[0][j], g[1 + q][j]);
+    dn[q] = fmaf(G[q][0], n[0], fmaf(G[q][1], n[1], G[q][2] * n[2]));
   }
-  Fv[4] = work + c.kap * c.gm1_over_R * qn;
+  const float tdiv = (2.f / 3.f) * (G[0][0] + G[1][1] + G[2][2]);
+  const float mr = c.mu * ir;
+  Fv[0] = 0.f;
+#pragma unroll
+  for (int q = 0; q < 3; q++)
+    Fv[1 + q] = mr * fmaf(G[0][q], n[0], fmaf(G[1][q], n[1], fmaf(G[2][q], n[2], fmaf(-tdiv, n[q], dn[q]))));
+  const float g0n = fmaf(g[0][0], n[0], fmaf(g[0][1], n[1], g[0][2] * n[2]));
+  const float e = ((c.H_ref - c.p_ref) + W[4]) * ir;
+  const float en = fmaf(-u[0], dn[0], fmaf(-u[1], dn[1], fmaf(-u[2], dn[2], fmaf(-e, g0n, g4n))));
+  Fv[4] = fmaf(u[0], Fv[1], fmaf(u[1], Fv[2], fmaf(u[2], Fv[3], c.k_e * ir * en)));
 }
 
 // value and gradient at (x, y, z) of a P3/P4 cell polynomial from its row
@@ -799,16 +777,20 @@ __global__ void __launch_bounds__(kFaceThreads, 1) k_face_mx(FaceArgsMx a) {
       // the viscous flux is linear in the gradient and scaling by 2 is exact, so
       // the flux of this gradient is exactly 2 F_v (and the halving of grad U_L +
       // grad U_R drops out)
-      float Wf[5], gf2[5][3];
+      float Wf[5], gf2[4][3];
 #pragma unroll
-      for (int v = 0; v < 5; v++) {
+      for (int v = 0; v < 4; v++) {
         const float jump2 = pen2 * (WR[v] - WL[v]);
         Wf[v] = 0.5f * (WL[v] + WR[v]);
 #pragma unroll
         for (int d = 0; d < 3; d++) gf2[v][d] = fmaf(jump2, n[d], gs[v][d]);
       }
+      Wf[4] = 0.5f * (WL[4] + WR[4]);
+      // the energy gradient enters through its normal part alone
+      const float g4n =
+          fmaf(gs[4][0], n[0], fmaf(gs[4][1], n[1], fmaf(gs[4][2], n[2], pen2 * (WR[4] - WL[4]))));
       float Fv2[5];
-      viscous_flux_mx(Wf, gf2, n, a.c, Fv2);
+      viscous_flux_mx(Wf, gf2, g4n, n, a.c, Fv2);
 #pragma unroll
       for (int v = 0; v < 5; v++) flux[v] = fmaf(-0.5f, Fv2[v], Fc[v]) * area;
     } else {
