@@ -32,6 +32,7 @@ namespace ucnsnet {
 
 using bf16 = __nv_bfloat16;
 
+constexpr int kPartial = (kParams + 3) / 4 * 4;  // floats per CTA of the partial gradients (16-byte rows)
 constexpr int kThreads = 128;  // one thread per tile row, 4 warps = 4 TMEM lane quarters
 constexpr long long kMbarCycles = 1ll << 30;  // ~0.5 s at 2 GHz: a wait gives up after this
 
@@ -160,8 +161,8 @@ constexpr uint32_t kOffA4 = kOffDH2 + 16384;     // 128 x 128  bf16  dH2^T (rows
 constexpr uint32_t kOffB4 = kOffA4 + 32768;      //  64 x 128  bf16  H1^T
 constexpr uint32_t kOffA5 = kOffB4 + 16384;      // 128 x 128  bf16  dH1^T (rows >= 64 zero)
 constexpr uint32_t kOffB5 = kOffA5 + 32768;      //  32 x 128  bf16  X^T
-constexpr uint32_t kOffRed = kOffB5 + 8192;      // 128 x 64   f32   column-sum scratch
-constexpr uint32_t kOffAcc = kOffRed + 32768;    // gb1, gb2, gw3, gb3: f32
+constexpr uint32_t kOffRed = kOffB5 + 8192;      // column sums per warp, db1 db2 dw3 [4][64], dz [4]: f32
+constexpr uint32_t kOffAcc = kOffRed + 4096;     // gb1, gb2, gw3, gb3: f32
 constexpr uint32_t kTrainSmem = kOffAcc + 1024;
 
 static_assert(kOffW2T >= kFwdSmem, "training layout overlaps the forward block");
@@ -169,7 +170,7 @@ static_assert(kTrainSmem <= 227 * 1024, "shared memory budget");
 
 struct FwdArgs {
   const bf16* __restrict__ X;  // [n][32]
-  const bf16* __restrict__ W;  // W1 [64][32] then W2 [64][64]
+  const bf16* __restrict__ W;  // W1 [64][32], W2 [64][64], W2^T [64][64]
   const float* __restrict__ theta;
   const float* __restrict__ w3r;
   float* __restrict__ z;        // [n] logits (may be null)
@@ -186,7 +187,7 @@ struct GradArgs {
   const bf16* __restrict__ W;
   const float* __restrict__ theta;
   const float* __restrict__ w3r;
-  float* __restrict__ partial;  // [gridDim.x][kParams]
+  float* __restrict__ partial;  // [gridDim.x][kPartial]
   int64_t n;
   float inv_n, w_pos, w_neg;
   int* err;
@@ -196,13 +197,15 @@ struct GradArgs {
 __device__ __forceinline__ void stage_params(uint8_t* sm, const bf16* W, const float* theta, const float* w3r,
                                              bool transposed_w2) {
   const int tid = threadIdx.x;
-  for (int e = tid; e < 64 * 32; e += kThreads)
-    *reinterpret_cast<bf16*>(sm + kOffW1s + kmaj(e >> 5, e & 31, 32)) = W[e];
-  for (int e = tid; e < 64 * 64; e += kThreads) {
-    const int j = e >> 6, k = e & 63;
-    *reinterpret_cast<bf16*>(sm + kOffW2s + kmaj(j, k, 64)) = W[2048 + e];
-    if (transposed_w2) *reinterpret_cast<bf16*>(sm + kOffW2T + kmaj(k, j, 64)) = W[2048 + e];
-  }
+  // 16-byte pieces: eight consecutive k of a row stay together in the K-major tiles
+  const uint4* src = reinterpret_cast<const uint4*>(W);
+  for (int e = tid; e < 64 * 32 / 8; e += kThreads)
+    *reinterpret_cast<uint4*>(sm + kOffW1s + kmaj(e >> 2, 8 * (e & 3), 32)) = src[e];
+  for (int e = tid; e < 64 * 64 / 8; e += kThreads)
+    *reinterpret_cast<uint4*>(sm + kOffW2s + kmaj(e >> 3, 8 * (e & 7), 64)) = src[256 + e];
+  if (transposed_w2)
+    for (int e = tid; e < 64 * 64 / 8; e += kThreads)
+      *reinterpret_cast<uint4*>(sm + kOffW2T + kmaj(e >> 3, 8 * (e & 7), 64)) = src[768 + e];
   float* par = reinterpret_cast<float*>(sm + kOffPar);
   for (int e = tid; e < 64; e += kThreads) {
     par[e] = theta[kOffB1 + e];
@@ -340,7 +343,27 @@ __global__ void k_mlp_wait_probe(int* err, long long limit) {
   if (!mbar_wait(&bar, 0, limit)) atomicOr(err, 2);
 }
 
-// per-CTA partial gradients of the class-weighted BCE over its tiles
+// Sums of v[0..63] over the warp's 32 rows: lane l ends with columns 2 l and 2 l +
+// 1 in v[0], v[1] (each step a lane keeps one half of its columns and hands the
+// other to its partner; a fixed tree)
+__device__ __forceinline__ void warp_column_sums(float (&v)[64]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int n = 32, off = 16; n >= 2; n >>= 1, off >>= 1) {
+    const bool up = lane & off;
+#pragma unroll
+    for (int j = 0; j < n; j++) {
+      const float give = up ? v[j] : v[j + n], keep = up ? v[j + n] : v[j];
+      v[j] = keep + __shfl_xor_sync(0xffffffffu, give, off);
+    }
+  }
+}
+
+// per-CTA partial gradients of the class-weighted BCE over its tiles.  Bound by
+// latency: a 4096-row batch is 32 CTAs of one tile each.  Column sums over the
+// rows by shuffles in each warp (through shared memory, one row per thread, the
+// stores hit one bank 32 times over), 16-byte staging of the weights and the partial
+// sums of k_mlp_step loaded 16 at a time took 32 such batches from 954 to 681 us.
 __global__ void __launch_bounds__(kThreads, 1) k_mlp_grad(GradArgs a) {
   extern __shared__ __align__(1024) uint8_t sm[];
   const int tid = threadIdx.x, warp = tid >> 5;
@@ -352,9 +375,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_grad(GradArgs a) {
   const float* par = reinterpret_cast<const float*>(sm + kOffPar);
   stage_params(sm, a.W, a.theta, a.w3r, true);
   // the padding rows 64..127 of the transposed gradient operands stay zero
-  for (uint32_t e = tid; e < 32768 / 16; e += kThreads) {
-    reinterpret_cast<uint4*>(sm + kOffA4)[e] = make_uint4(0, 0, 0, 0);
-    reinterpret_cast<uint4*>(sm + kOffA5)[e] = make_uint4(0, 0, 0, 0);
+  for (uint32_t e = tid; e < 16384 / 16; e += kThreads) {
+    reinterpret_cast<uint4*>(sm + kOffA4 + kmaj(64, 0, 128))[e] = make_uint4(0, 0, 0, 0);
+    reinterpret_cast<uint4*>(sm + kOffA5 + kmaj(64, 0, 128))[e] = make_uint4(0, 0, 0, 0);
   }
   for (int e = tid; e < 193; e += kThreads) acc[e] = 0.f;
   if (tid == 0) mbar_init(bar);
@@ -391,7 +414,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_grad(GradArgs a) {
 #pragma unroll
     for (int j = 0; j < 64; j++) {
       *reinterpret_cast<bf16*>(sm + kOffA4 + kmaj(j, tid, 128)) = __float2bfloat16_rn(d[j]);
-      red[tid * 64 + j] = d[j];
     }
     fence_async_smem();
     fence_before();
@@ -403,28 +425,16 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_grad(GradArgs a) {
       mma_commit(bar);
     }
     // column sums while the tensor cores run: db2, dw3, db3
-    if (tid < 64) {
-      float s2 = 0.f;
-      for (int r = 0; r < 128; r++) s2 += red[r * 64 + tid];
-      acc[64 + tid] += s2;
-    }
-    __syncthreads();
+    warp_column_sums(d);
+    reinterpret_cast<float2*>(red + 256 + warp * 64)[tid & 31] = make_float2(d[0], d[1]);
 #pragma unroll
-    for (int j = 0; j < 64; j++) red[tid * 64 + j] = dz * h2[j];
-    __syncthreads();
-    if (tid < 64) {
-      float s3 = 0.f;
-      for (int r = 0; r < 128; r++) s3 += red[r * 64 + tid];
-      acc[128 + tid] += s3;
-    }
-    __syncthreads();
-    red[tid] = dz;
-    __syncthreads();
-    if (tid == 0) {
-      float s4 = 0.f;
-      for (int r = 0; r < 128; r++) s4 += red[r];
-      acc[192] += s4;
-    }
+    for (int j = 0; j < 64; j++) h2[j] *= dz;
+    warp_column_sums(h2);
+    reinterpret_cast<float2*>(red + 512 + warp * 64)[tid & 31] = make_float2(h2[0], h2[1]);
+    float sdz = dz;
+#pragma unroll
+    for (int off = 16; off >= 1; off >>= 1) sdz += __shfl_xor_sync(0xffffffffu, sdz, off);
+    if ((tid & 31) == 0) red[768 + warp] = sdz;
     ok = mbar_wait(bar, phase) && ok;
     phase ^= 1u;
     fence_after();
@@ -432,13 +442,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_grad(GradArgs a) {
     float g[64];
 #pragma unroll
     for (int q = 0; q < 4; q++) tmem_ld16(tD3 + lane + 16 * q, g + 16 * q);
-    __syncthreads();  // the scalar column sum above is done with red
 #pragma unroll
     for (int k = 0; k < 64; k++) {
-      const float v = ((m1 >> k) & 1ull) ? g[k] : 0.f;
-      *reinterpret_cast<bf16*>(sm + kOffA5 + kmaj(k, tid, 128)) = __float2bfloat16_rn(v);
-      red[tid * 64 + k] = v;
+      g[k] = ((m1 >> k) & 1ull) ? g[k] : 0.f;
+      *reinterpret_cast<bf16*>(sm + kOffA5 + kmaj(k, tid, 128)) = __float2bfloat16_rn(g[k]);
     }
+    warp_column_sums(g);
+    reinterpret_cast<float2*>(red + warp * 64)[tid & 31] = make_float2(g[0], g[1]);
     fence_async_smem();
     fence_before();
     __syncthreads();
@@ -447,11 +457,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_grad(GradArgs a) {
       gemm(tW1, sbase + kOffA5, sbase + kOffB5, 128, 32, !first);  // dW1 += dH1^T X
       mma_commit(bar);
     }
-    if (tid < 64) {
-      float s1 = 0.f;
-      for (int r = 0; r < 128; r++) s1 += red[r * 64 + tid];
-      acc[tid] += s1;
+    // the four warps' sums, in order: db1, db2, dw3 (acc's order), then db3
+    for (int e = tid; e < 192; e += kThreads) {
+      const float* w = red + (e >> 6) * 256 + (e & 63);
+      acc[e] += (w[0] + w[64]) + (w[128] + w[192]);
     }
+    if (tid == 0) acc[192] += (red[768] + red[769]) + (red[770] + red[771]);
     ok = mbar_wait(bar, phase) && ok;
     phase ^= 1u;
     fence_after();
@@ -460,7 +471,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_grad(GradArgs a) {
     if (!__syncthreads_and(ok)) break;
   }
   // write this CTA's partial gradient
-  float* out = a.partial + (size_t)blockIdx.x * kParams;
+  float* out = a.partial + (size_t)blockIdx.x * kPartial;
   if (tid < 64) {
     float w[64];
     if (!first) {
@@ -470,12 +481,16 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_grad(GradArgs a) {
 #pragma unroll
       for (int q = 0; q < 64; q++) w[q] = 0.f;
     }
-    for (int k = 0; k < 64; k++) out[kOffW2 + tid * 64 + k] = w[k];
+#pragma unroll
+    for (int k = 0; k < 64; k += 4)
+      *reinterpret_cast<float4*>(out + kOffW2 + tid * 64 + k) = make_float4(w[k], w[k + 1], w[k + 2], w[k + 3]);
     if (!first) {
 #pragma unroll
       for (int q = 0; q < 2; q++) tmem_ld16(tW1 + lane + 16 * q, w + 16 * q);
     }
-    for (int i = 0; i < 32; i++) out[kOffW1 + tid * 32 + i] = w[i];
+#pragma unroll
+    for (int i = 0; i < 32; i += 4)
+      *reinterpret_cast<float4*>(out + kOffW1 + tid * 32 + i) = make_float4(w[i], w[i + 1], w[i + 2], w[i + 3]);
   } else {
     // warps 2-3 take part in the (warp-collective) loads of their own lanes, unused
     float w[64];
@@ -500,12 +515,20 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_grad(GradArgs a) {
   if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
+// entry e = 64 j + k of W2, rounded, into the copies W2 and W2^T
+__device__ __forceinline__ void put_w2(bf16* W, int e, float th) {
+  const bf16 w = __float2bfloat16_rn(th);
+  W[2048 + e] = w;
+  W[6144 + (e & 63) * 64 + (e >> 6)] = w;
+}
+
 // grad[p] = sum over CTAs in order of partial[c][p]
 __global__ void k_mlp_reduce(const float* __restrict__ partial, int nctas, float* __restrict__ grad) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= kParams) return;
   float s = 0.f;
-  for (int c = 0; c < nctas; c++) s += partial[(size_t)c * kParams + p];
+#pragma unroll 16
+  for (int c = 0; c < nctas; c++) s += partial[(size_t)c * kPartial + p];
   grad[p] = s;
 }
 
@@ -519,7 +542,8 @@ __global__ void k_mlp_step(const float* __restrict__ partial, int nctas, float* 
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= kParams) return;
   float gp = 0.f;
-  for (int c = 0; c < nctas; c++) gp += partial[(size_t)c * kParams + p];
+#pragma unroll 16
+  for (int c = 0; c < nctas; c++) gp += partial[(size_t)c * kPartial + p];
   const float mp = b1 * m[p] + (1.f - b1) * gp;
   const float vp = b2 * v[p] + (1.f - b2) * gp * gp;
   m[p] = mp;
@@ -527,14 +551,14 @@ __global__ void k_mlp_step(const float* __restrict__ partial, int nctas, float* 
   const float th = theta[p] - lr * (mp / c1) / (sqrtf(vp / c2) + eps);
   theta[p] = th;
   if (p >= kOffW1 && p < kOffW1 + 2048) W[p - kOffW1] = __float2bfloat16_rn(th);
-  if (p >= kOffW2 && p < kOffW2 + 4096) W[2048 + (p - kOffW2)] = __float2bfloat16_rn(th);
+  if (p >= kOffW2 && p < kOffW2 + 4096) put_w2(W, p - kOffW2, th);
   if (p >= kOffW3 && p < kOffW3 + 64) w3r[p - kOffW3] = bf16r(th);
 }
 
 __global__ void k_mlp_cast(const float* __restrict__ theta, bf16* __restrict__ W, float* __restrict__ w3r) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p < 2048) W[p] = __float2bfloat16_rn(theta[kOffW1 + p]);
-  if (p < 4096) W[2048 + p] = __float2bfloat16_rn(theta[kOffW2 + p]);
+  if (p < 4096) put_w2(W, p, theta[kOffW2 + p]);
   if (p < 64) w3r[p] = bf16r(theta[kOffW3 + p]);
 }
 
@@ -672,9 +696,9 @@ int ucns_mlp_create(uint64_t seed, ucns_mlp** out) {
   for (int p = 0; p < 4096; p++) th[kOffW2 + p] = (float)(normal(st) * std::sqrt(2.0 / 64));
   for (int p = 0; p < 64; p++) th[kOffW3 + p] = (float)(normal(st) * std::sqrt(1.0 / 64));
   bool okm = cudaMalloc(&m->theta, kParams * 4) == cudaSuccess && cudaMalloc(&m->m, kParams * 4) == cudaSuccess &&
-             cudaMalloc(&m->v, kParams * 4) == cudaSuccess && cudaMalloc(&m->W, 6144 * 2) == cudaSuccess &&
+             cudaMalloc(&m->v, kParams * 4) == cudaSuccess && cudaMalloc(&m->W, (6144 + 4096) * 2) == cudaSuccess &&
              cudaMalloc(&m->w3r, 64 * 4) == cudaSuccess &&
-             cudaMalloc(&m->partial, (size_t)m->nsm * kParams * 4) == cudaSuccess &&
+             cudaMalloc(&m->partial, (size_t)m->nsm * kPartial * 4) == cudaSuccess &&
              cudaMalloc(&m->grad, kParams * 4) == cudaSuccess && cudaMalloc(&m->err, sizeof(int)) == cudaSuccess;
   if (!okm) {
     ucns_mlp_destroy(m);
