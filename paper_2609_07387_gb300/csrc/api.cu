@@ -112,6 +112,40 @@ int upload_fx_tiles(const ucns_mesh* m, const HostArrays& h, unsigned char** dst
   return upload(dst, b);
 }
 
+// The FP64 face geometry from P2 on: per cell the exponents of its axis scales (the
+// powers of two above the largest |offset| of its face points along each axis),
+// and the offsets of fq as fixed-point limb pairs in those units
+int upload_fixed_faces(const ucns_mesh* m, double** dst, int16_t** dst_h, const std::vector<double>& fq) {
+  const std::vector<int32_t>&fo = m->fo, &fn = m->fn;
+  const int64_t F = m->F, N = m->N;
+  const int nq = m->nq;
+  std::vector<int16_t> h((size_t)N * 4, 0);
+#pragma omp parallel for schedule(static)
+  for (int64_t i = 0; i < N; i++)
+    for (int d = 0; d < 3; d++) {
+      double big = 0.0;
+      for (int lf = 0; lf < m->nfc; lf++) {
+        const int32_t e = m->cf[(size_t)i * m->nfc + lf];
+        for (int q = 0; q < nq; q++)
+          big = std::fmax(big, std::fabs(fq[((size_t)q * 10 + d + (e & 1 ? 3 : 0)) * F + (e >> 1)]));
+      }
+      h[(size_t)i * 4 + d] = (int16_t)fx_row_exponent(big);
+    }
+  std::vector<double> g(fq);
+  for (int q = 0; q < nq; q++)
+    for (int c = 0; c < 6; c++) {
+      double* row = &g[((size_t)q * 10 + c) * F];
+#pragma omp parallel for schedule(static)
+      for (int64_t f = 0; f < F; f++) {
+        const int32_t i = c < 3 ? fo[f] : fn[f];
+        const int2 w = i < 0 ? make_int2(0, 0) : fx_limbs(fx_round(std::ldexp(row[f], 58 - h[(size_t)i * 4 + c % 3])));
+        std::memcpy(&row[f], &w, sizeof w);
+      }
+    }
+  int rc = upload(dst, g);
+  return rc ? rc : upload(dst_h, h);
+}
+
 template <typename T>
 int alloc(T** dst, size_t n) {
   if (cudaMalloc((void**)dst, n * sizeof(T)) != cudaSuccess)
@@ -380,7 +414,9 @@ int launch_recon_ho(ucns_mesh* m, const double* U, cudaStream_t s) {
   a.Msi = m->d.Msi;
   a.psib = m->d.psib;
   a.inv_h = m->d.inv_h;
+  a.hexp = reinterpret_cast<const short4*>(m->d.hexp);
   a.coef = m->d.coef;
+  a.cexp = m->d.cexp;
   a.N = (int)m->N;
   const double lsum = m->P.lambda_central + m->nd;
   a.lam0 = m->P.lambda_central / lsum;
@@ -402,6 +438,8 @@ int launch_recon_ho(ucns_mesh* m, const double* U, cudaStream_t s) {
 int launch_face_ho(ucns_mesh* m, cudaStream_t s) {
   FaceArgs a;
   a.coef = m->d.coef;
+  a.cexp = m->d.cexp;
+  a.hexp = reinterpret_cast<const short4*>(m->d.hexp);
   a.fq = m->d.fq;
   a.fpen = m->d.fpen;
   a.fo = m->d.fo;
@@ -414,13 +452,13 @@ int launch_face_ho(ucns_mesh* m, cudaStream_t s) {
   const bool visc = m->P.reynolds > 0.0;
   const int fpw = 32 / m->nq;  // faces per warp
   const size_t threads = (size_t)((m->F + fpw - 1) / fpw) * 32;
-  const unsigned g = nblocks(threads, 128);
+  const unsigned g = nblocks(threads, kFaceHoThreads);
   if (m->K == 19) {
-    if (visc) k_face_ho<3, true><<<g, 128, 0, s>>>(a);
-    else k_face_ho<3, false><<<g, 128, 0, s>>>(a);
+    if (visc) k_face_ho<3, true><<<g, kFaceHoThreads, 0, s>>>(a);
+    else k_face_ho<3, false><<<g, kFaceHoThreads, 0, s>>>(a);
   } else {
-    if (visc) k_face_ho<4, true><<<g, 128, 0, s>>>(a);
-    else k_face_ho<4, false><<<g, 128, 0, s>>>(a);
+    if (visc) k_face_ho<4, true><<<g, kFaceHoThreads, 0, s>>>(a);
+    else k_face_ho<4, false><<<g, kFaceHoThreads, 0, s>>>(a);
   }
   UCNS_CUDA(cudaGetLastError());
   return UCNS_OK;
@@ -448,7 +486,9 @@ int launch_recon_raw(ucns_mesh* m, const double* U, cudaStream_t s) {
   a.err = m->d.err;
   a.mom = m->d.mom;
   a.inv_h = m->d.inv_h;
+  a.hexp = reinterpret_cast<const short4*>(m->d.hexp);
   a.coef = m->d.coef;
+  a.cexp = m->d.cexp;
   a.gate = m->gate_eval_active ? m->gate_flag : nullptr;
   a.dev = m->label_out;
   a.dvalid = m->d.dvalid;
@@ -479,6 +519,8 @@ int launch_face_raw(ucns_mesh* m, cudaStream_t s) {
   if (m->K > 9) return launch_face_ho(m, s);
   FaceArgs a;
   a.coef = m->d.coef;
+  a.cexp = m->d.cexp;
+  a.hexp = reinterpret_cast<const short4*>(m->d.hexp);
   a.fq = m->d.fq;
   a.fpen = m->d.fpen;
   a.fo = m->d.fo;
@@ -741,6 +783,14 @@ int residual_into(ucns_mesh* m, const double* U, double* R, cudaStream_t s) {
   return UCNS_OK;
 }
 
+// the FP64 form's diagnostic partials, from the coefficients of the last reconstruction
+void launch_diag_partial(ucns_mesh* m, const double* U, cudaStream_t s) {
+  const int order = m->K == 3 ? 1 : (m->K == 9 ? 2 : (m->K == 19 ? 3 : 4));
+  k_diag_partial<<<m->d.red_blocks, kRedThreads, 0, s>>>(U, m->d.coef, m->d.cexp,
+                                                         reinterpret_cast<const short4*>(m->d.hexp),
+                                                         fx_coef_bits(order), m->d.vol, (int)m->N, m->d.red);
+}
+
 // Diagnostic sums [V KE, V |curl u|^2, V (div u)^2, V] of the coefficients
 // the last reconstruction left, into out[0..3] (device)
 int diag_sums_into(ucns_mesh* m, const double* U, double* out, cudaStream_t s) {
@@ -748,7 +798,7 @@ int diag_sums_into(ucns_mesh* m, const double* U, double* out, cudaStream_t s) {
     k_diag_partial_mx<<<m->d.red_blocks, kRedThreads, 0, s>>>(U, m->d.coeff, coef_row_floats(m), m->NC, m->d.vol,
                                                              (int)m->N, m->d.red);
   else
-    k_diag_partial<double><<<m->d.red_blocks, kRedThreads, 0, s>>>(U, m->d.coef, m->d.vol, (int)m->N, m->d.red);
+    launch_diag_partial(m, U, s);
   k_sum_partials<<<1, 32 * 4, 0, s>>>(m->d.red, m->d.red_blocks, 4, 4, out);
   UCNS_CUDA(cudaGetLastError());
   return UCNS_OK;
@@ -910,7 +960,7 @@ void device_free(ucns_mesh* m) {
   m->gate_eval_active = false;
   m->gate_fixed = false;
   DeviceMesh& d = m->d;
-  void* ptrs[] = {d.fslot, d.bcell, d.bcount, d.inv_vol, d.vol, d.inv_h, d.dtlen, d.mom, d.sc, d.Pc, d.sd, d.Pd, d.fxt, d.Msi, d.psib, d.hot, d.Msif, d.psibf, d.Pcb, d.Pdb, d.scb, d.sdb, d.cellb, d.sda, d.Pda,
+  void* ptrs[] = {d.fslot, d.bcell, d.bcount, d.inv_vol, d.vol, d.inv_h, d.dtlen, d.mom, d.sc, d.Pc, d.sd, d.Pd, d.fxt, d.hexp, d.cexp, d.Msi, d.psib, d.hot, d.Msif, d.psibf, d.Pcb, d.Pdb, d.scb, d.sdb, d.cellb, d.sda, d.Pda,
                   d.inv_hf, d.fpenf, d.cf, d.fo, d.fn, d.dvalid, d.fq, d.fqf, d.fpen, d.coef, d.coeff, d.Uhl, d.G,
                   d.Ustage, d.Uacc, d.Uhost, d.red, d.dt, d.err, d.dt_part, d.dt_count};
   for (void* p : ptrs)
@@ -1146,7 +1196,10 @@ static int device_upload(ucns_mesh* m, const ucns_params* p, const HostArrays& h
       return rc;
     }
   } else if ((m->K == 9 && (rc = upload_fx_tiles(m, h, &d.fxt))) ||
-             (m->K != 9 && ((rc = upload(&d.Pc, h.Pc)) || (rc = upload(&d.Pd, h.Pd)))) || (rc = upload(&d.fq, h.fq)) ||
+             (m->K != 9 && ((rc = upload(&d.Pc, h.Pc)) || (rc = upload(&d.Pd, h.Pd)))) ||
+             (m->K == 3 && (rc = upload(&d.fq, h.fq))) ||
+             (m->K > 3 && ((rc = upload_fixed_faces(m, &d.fq, &d.hexp, h.fq)) ||
+                            (rc = alloc(&d.cexp, (size_t)5 * m->N)))) ||
              (rc = upload(&d.fpen, h.fpen)) || (rc = upload(&d.Msi, h.Msi)) || (rc = upload(&d.psib, h.psib)) ||
              (rc = alloc(&d.coef, (size_t)m->NC * m->N * 5))) {
     device_free(m);
@@ -1348,7 +1401,7 @@ int ucns_diagnostics(ucns_mesh* m, const double* U, ucns_diag* out, void* stream
       k_diag_partial_mx<<<m->d.red_blocks, kRedThreads, 0, s>>>(U, m->d.coeff, coef_row_floats(m), m->NC,
                                                                  m->d.vol, (int)m->N, m->d.red);
     else
-      k_diag_partial<double><<<m->d.red_blocks, kRedThreads, 0, s>>>(U, m->d.coef, m->d.vol, (int)m->N, m->d.red);
+      launch_diag_partial(m, U, s);
     // the final sums land in the first 4 doubles of G (free between residuals)
     k_sum_partials<<<1, 32 * 4, 0, s>>>(m->d.red, m->d.red_blocks, 4, 4, m->d.G);
     UCNS_CUDA(cudaGetLastError());

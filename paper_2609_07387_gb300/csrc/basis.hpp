@@ -30,4 +30,16 @@ UCNS_HD constexpr int basis_exp(int k, int d) {
 
 UCNS_HD constexpr int basis_degree(int k) { return basis_exp(k, 0) + basis_exp(k, 1) + basis_exp(k, 2); }
 
+// the mode with exponents (a, b, c), of degree 1 or more
+UCNS_HD constexpr int basis_index(int a, int b, int c) {
+  const int deg = a + b + c, i = b + c;
+  if (deg == 2) return a == 2 ? 3 : (b == 2 ? 4 : (c == 2 ? 5 : (c == 0 ? 6 : (b == 0 ? 7 : 8))));
+  return basis_count(deg - 1) + i * (i + 1) / 2 + (i - b);
+}
+
+// the mode of basis monomial k divided by coordinate d (k of degree 2 or more, with exponent of d at least 1)
+UCNS_HD constexpr int basis_lower(int k, int d) {
+  return basis_index(basis_exp(k, 0) - (d == 0), basis_exp(k, 1) - (d == 1), basis_exp(k, 2) - (d == 2));
+}
+
 }  // namespace ucns

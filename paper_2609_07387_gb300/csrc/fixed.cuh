@@ -14,6 +14,9 @@
 //   operands     |q| <= 2^B, B = 58 (57 in sums of more than 38): d = q
 //                2^(e - B), |d| < 2^e for all d of the sum
 //   monomials    |q| <= 2^58: x = q 2^-58, |x| <= 1
+//   polynomials  coefficients as operands (B = 58, 57 at P4), aligned to the
+//                largest of the cell's in coordinates scaled by powers of two,
+//                one per axis, to [-1, 1]
 // A product is (hi hi') 2^60 + (hi lo' + lo hi') 2^30 + lo lo'; the last term,
 // at most 2^58, is dropped.  Bounds: sum |hi hi'| <= 2^30 2^28, sum |hi lo' + lo
 // hi'| <= 2^30 2^29 + M 2^29 2^(B - 30) < 2^63, so no accumulator overflows for
@@ -54,10 +57,20 @@ struct FxAcc {
   long long h = 0, m = 0;
 };
 
+// a += x y, one instruction (written as an expression, the compiler rearranges
+// sums of products into trees of 64-bit additions, two more instructions each)
+__host__ __device__ __forceinline__ void fx_wide(long long& a, int x, int y) {
+#ifdef __CUDA_ARCH__
+  asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(a) : "r"(x), "r"(y));
+#else
+  a += (long long)x * y;
+#endif
+}
+
 __host__ __device__ __forceinline__ void fx_mac(FxAcc& a, int2 p, int2 d) {
-  a.h += (long long)p.x * d.x;
-  a.m += (long long)p.x * d.y;
-  a.m += (long long)p.y * d.x;
+  fx_wide(a.h, p.x, d.x);
+  fx_wide(a.m, p.x, d.y);
+  fx_wide(a.m, p.y, d.x);
 }
 
 // the sum in units of 2^58 (|h| < 2^61)
@@ -180,5 +193,41 @@ __host__ __device__ __forceinline__ void fx_differences(double (&u)[M], double u
   for (int m = 0; m < M; m++) q[m] = fx_limbs(((d[m] << (lz - 1)) + (1ll << (62 - B))) >> (63 - B));
   e = eb == 2047 ? kFxNan : eb - 1020 - lz - low;
 }
+
+// The same for polynomial coefficients d[k], each to be scaled by 2^off[k].
+template <int M>
+__host__ __device__ __forceinline__ int fx_align_scaled(double (&d)[M], const int (&off)[M], int& e) {
+  bool bad = false;
+  int eb = -(1 << 14);
+#pragma unroll
+  for (int m = 0; m < M; m++) {
+    const int x = fx_exponent(d[m]);
+    bad = bad || x == 2047;
+    eb = x + off[m] > eb ? x + off[m] : eb;
+  }
+  e = eb - 1022;
+  if (eb < 64) {
+    eb = -(1 << 14);
+#pragma unroll
+    for (int m = 0; m < M; m++) {
+      d[m] *= 0x1p512;
+      const int x = fx_exponent(d[m]);
+      eb = x + off[m] > eb ? x + off[m] : eb;
+    }
+    e = eb - 1022 - 512;
+  }
+  if (bad) e = kFxNan;
+  return eb;
+}
+
+// product of two monomials
+__host__ __device__ __forceinline__ int2 fx_mul(int2 a, int2 b) {
+  FxAcc t;
+  fx_mac(t, a, b);
+  return fx_limbs(fx_sum(t));
+}
+
+// the integer hi 2^30 + lo
+__host__ __device__ __forceinline__ long long fx_value(int2 q) { return ((long long)q.x << 30) + q.y; }
 
 }  // namespace ucns

@@ -15,6 +15,7 @@
 
 #include <cstdint>
 
+#include "basis.hpp"
 #include "bulk.cuh"
 #include "fixed.cuh"
 
@@ -31,7 +32,10 @@ struct ReconArgs {
   const unsigned char* __restrict__ tiles;  // per 32-cell tile its stencils and least-squares rows (P2, FxTile)
   const double* __restrict__ mom;  // [6][N]
   const double* __restrict__ inv_h;  // [N]
-  double* __restrict__ coef;       // [NC][N][5] physical-unit monomial coefficients
+  const short4* __restrict__ hexp; // [N] exponents of the cell's axis scales (from P2 on)
+  double* __restrict__ coef;       // [NC][N][5] physical-unit monomial coefficients; from P2 on the
+                                   // non-constant ones in fixed point, (hi, lo) limb pairs in place of the doubles
+  int32_t* __restrict__ cexp;      // [N][5] their exponents (from P2 on)
   const uint8_t* __restrict__ gate;  // [N]: 0 -> linear weights (null: every cell CWENOZ)
   float* __restrict__ dev;           // [N]: max |omega - lambda| (null: not wanted)
   const uint8_t* __restrict__ dvalid;  // [N] bit s: directional candidate s exists (WALLS kernels)
@@ -64,7 +68,11 @@ static_assert(FxTile::CENTRAL % 16 == 0 && FxTile::directional(4) % 16 == 0 && F
 
 struct FaceArgs {
   const double* __restrict__ coef;
-  const double* __restrict__ fq;  // [nq][10][F]: x - x_L, x - x_R' (physical), n, |dS|
+  const int32_t* __restrict__ cexp;  // [N][5] (from P2 on)
+  const short4* __restrict__ hexp;   // [N] (from P2 on)
+  // [nq][10][F]: x - x_L, x - x_R', n, |dS|; the offsets physical (P1), or in
+  // fixed point and in units of the axis scales of their cell (from P2 on)
+  const double* __restrict__ fq;
   const double* __restrict__ fpen;
   const int32_t* __restrict__ fo;
   const int32_t* __restrict__ fn;
@@ -242,6 +250,27 @@ __device__ __forceinline__ void fx_contract(const double* __restrict__ Uv, doubl
   }
 }
 
+// bits of the polynomial coefficients in fixed point
+__host__ __device__ constexpr int fx_coef_bits(int order) { return order == 4 ? 57 : 58; }
+
+// The coefficients c of the monomials in x - x_i (physical) as the face kernels
+// read them: scaled by the cell's axis scales H_d = 2^h_d, at least the largest
+// |x_d - x_i,d| of its face points, aligned to the largest and split into limbs
+template <int ORDER>
+__device__ __forceinline__ void store_fixed(double (&c)[basis_count(ORDER)], short4 h, double* out, size_t st,
+                                            int32_t* cexp) {
+  constexpr int K = basis_count(ORDER);
+  int off[K];
+#pragma unroll
+  for (int k = 0; k < K; k++) off[k] = basis_exp(k, 0) * h.x + basis_exp(k, 1) * h.y + basis_exp(k, 2) * h.z;
+  int e;
+  const int eb = fx_align_scaled<K>(c, off, e);
+#pragma unroll
+  for (int k = 0; k < K; k++)
+    *reinterpret_cast<int2*>(out + (k + 1) * st) = fx_operand<fx_coef_bits(ORDER)>(c[k], eb - off[k]);
+  *cexp = e;
+}
+
 // P1: thread = (cell i, variable v), tid = 5 i + v
 __global__ void __launch_bounds__(256) k_recon_p1(ReconArgs a) {
   const int tid = blockIdx.x * blockDim.x + threadIdx.x;
@@ -274,7 +303,8 @@ __global__ void __launch_bounds__(256) k_recon_p1(ReconArgs a) {
 // the pipe's FMA rate.  Contractions in integers from global memory 1970 us (the
 // loads' latency at 12 warps per SM), from shared memory tiles 1648, with the
 // differences in integers too and one division for all weights 1192 (3, 4, 5
-// blocks per SM: 1210, 1192, 1229).
+// blocks per SM: 1210, 1192, 1229), with single-instruction accumulation and
+// coefficients written in fixed point 1060.
 template <bool WENO, int ND, bool GATED, bool WALLS = false>
 __global__ void __launch_bounds__(FxTile::THREADS, 4) k_recon(ReconArgs a) {
   using T = FxTile;
@@ -449,46 +479,97 @@ __global__ void __launch_bounds__(FxTile::THREADS, 4) k_recon(ReconArgs a) {
   const size_t st = (size_t)N * 5;
   out[0] = c0;
 #pragma unroll
-  for (int k = 0; k < K; k++) out[(k + 1) * st] = cf[k] * (k < 3 ? ih : ih2);
+  for (int k = 0; k < K; k++) cf[k] *= k < 3 ? ih : ih2;
+  store_fixed<2>(cf, a.hexp[i], out, st, a.cexp + (size_t)i * 5 + v);
 }
 
 // ----------------------------------------------------------- face flux
-// value at the physical offset (x, y, z) from the centroid into U; gradient
+// P1: value at the physical offset (x, y, z) from the centroid into U; gradient
 // written (ACC = false) or added (ACC = true) into g
-template <int ORDER, bool ACC>
-__device__ __forceinline__ void eval_side(const double* __restrict__ coef, int N, int cell,
-                                          double x, double y, double z, double U[5], double g[5][3]) {
+template <bool ACC>
+__device__ __forceinline__ void eval_side_p1(const double* __restrict__ coef, int N, int cell,
+                                             double x, double y, double z, double U[5], double g[5][3]) {
   const size_t st = (size_t)N * 5;
   const double* p = coef + (size_t)cell * 5;
 #pragma unroll
   for (int v = 0; v < 5; v++) {
     const double c0 = p[v], c1 = p[st + v], c2 = p[2 * st + v], c3 = p[3 * st + v];
-    double gx, gy, gz;
-    if (ORDER == 1) {
-      U[v] = fma(c1, x, fma(c2, y, fma(c3, z, c0)));
-      gx = c1;
-      gy = c2;
-      gz = c3;
-    } else {
-      const double c4 = p[4 * st + v], c5 = p[5 * st + v], c6 = p[6 * st + v];
-      const double c7 = p[7 * st + v], c8 = p[8 * st + v], c9 = p[9 * st + v];
-      const double tx = fma(c4, x, fma(c7, y, fma(c8, z, c1)));
-      const double ty = fma(c5, y, fma(c9, z, c2));
-      const double tz = fma(c6, z, c3);
-      U[v] = fma(x, tx, fma(y, ty, fma(z, tz, c0)));
-      gx = fma(c4, x, tx);                       // c1 + 2c4 x + c7 y + c8 z
-      gy = fma(c7, x, fma(c5, y, ty));           // c2 + c7 x + 2c5 y + c9 z
-      gz = fma(c8, x, fma(c9, y, fma(c6, z, tz)));  // c3 + c8 x + c9 y + 2c6 z
-    }
+    U[v] = fma(c1, x, fma(c2, y, fma(c3, z, c0)));
     if (ACC) {
-      g[v][0] += gx;
-      g[v][1] += gy;
-      g[v][2] += gz;
+      g[v][0] += c1;
+      g[v][1] += c2;
+      g[v][2] += c3;
     } else {
-      g[v][0] = gx;
-      g[v][1] = gy;
-      g[v][2] = gz;
+      g[v][0] = c1;
+      g[v][1] = c2;
+      g[v][2] = c3;
     }
+  }
+}
+
+// From P2 on: the same at the offset (x, y, z), fixed point in units of the cell's
+// axis scales: products and sums on the integer pipe (fixed.cuh), one rounding to
+// FP64 of each value and gradient component.  k_face<2> at 72 x 80 x 88, us: FP64
+// evaluation 4756 (165 of its 430 FP64 operations a point), this 3220 (the FP64 pipe
+// busy 85 %).
+template <int ORDER>
+struct FxPoint {
+  int2 m[basis_count(ORDER)];  // the monomials
+  __device__ __forceinline__ FxPoint(int2 x, int2 y, int2 z) {
+    m[0] = x;
+    m[1] = y;
+    m[2] = z;
+#pragma unroll
+    for (int k = 3; k < basis_count(ORDER); k++) {
+      const int d = basis_exp(k, 0) ? 0 : (basis_exp(k, 1) ? 1 : 2);
+      m[k] = fx_mul(m[basis_lower(k, d)], m[d]);
+    }
+  }
+  // value u and gradient g of one variable: p its constant term (the others st
+  // doubles apart each), e its exponent, h the cell's axis scales
+  __device__ __forceinline__ void eval(const double* p, size_t st, int e, short4 h, double& u, double (&g)[3]) const {
+    FxAcc a, s[3];
+    long long lin[3];
+#pragma unroll
+    for (int k = 0; k < basis_count(ORDER); k++) {
+      const int2 c = *reinterpret_cast<const int2*>(p + (k + 1) * st);
+      fx_mac(a, c, m[k]);
+      if (k < 3) {
+        lin[k] = fx_value(c);
+      } else {
+#pragma unroll
+        for (int d = 0; d < 3; d++) {
+          const int n = basis_exp(k, d);
+          if (n) {
+            // n times the monomial: |lo| <= 4 2^29, still an int
+            const int2 w = m[basis_lower(k, d)];
+            fx_mac(s[d], c, make_int2(n * w.x, n * w.y));
+          }
+        }
+      }
+    }
+    e -= fx_coef_bits(ORDER);
+    u = *p + fx_double(fx_sum(a), e);
+    const int hd[3] = {h.x, h.y, h.z};
+#pragma unroll
+    for (int d = 0; d < 3; d++) g[d] = fx_double(fx_sum(s[d]) + lin[d], e - hd[d]);
+  }
+};
+
+template <int ORDER, bool ACC>
+__device__ __forceinline__ void eval_side(const double* __restrict__ coef, const int32_t* __restrict__ cexp,
+                                          const short4* __restrict__ hexp, int N, int cell, int2 x, int2 y, int2 z,
+                                          double U[5], double g[5][3]) {
+  const size_t st = (size_t)N * 5;
+  const double* p = coef + (size_t)cell * 5;
+  const short4 h = __ldg(&hexp[cell]);
+  const FxPoint<ORDER> pt(x, y, z);
+#pragma unroll
+  for (int v = 0; v < 5; v++) {
+    double t[3];
+    pt.eval(p + v, st, cexp[(size_t)cell * 5 + v], h, U[v], t);
+#pragma unroll
+    for (int d = 0; d < 3; d++) g[v][d] = ACC ? g[v][d] + t[d] : t[d];
   }
 }
 
@@ -525,15 +606,20 @@ __global__ void __launch_bounds__(256) k_face(FaceArgs a) {
   const int fc = live ? f : a.F - 1;
   const size_t F = a.F;
   const double* __restrict__ fq = a.fq + (size_t)q * 10 * F + fc;
-  const double xl = fq[0], yl = fq[F], zl = fq[2 * F];
-  const double xr = fq[3 * F], yr = fq[4 * F], zr = fq[5 * F];
   const double n[3] = {fq[6 * F], fq[7 * F], fq[8 * F]};
   const double area = fq[9 * F];
   const int o = a.fo[fc], nb = a.fn[fc];
   double UL[5], UR[5], gs[5][3];  // gs = grad U_L + grad U_R
-  eval_side<ORDER, false>(a.coef, a.N, o, xl, yl, zl, UL, gs);
-  if (BND && nb < 0) ghost_state(-1 - nb, UL, n, a.uinf, UR);
-  else eval_side<ORDER, true>(a.coef, a.N, nb, xr, yr, zr, UR, gs);
+  if constexpr (ORDER == 1) {
+    eval_side_p1<false>(a.coef, a.N, o, fq[0], fq[F], fq[2 * F], UL, gs);
+    if (BND && nb < 0) ghost_state(-1 - nb, UL, n, a.uinf, UR);
+    else eval_side_p1<true>(a.coef, a.N, nb, fq[3 * F], fq[4 * F], fq[5 * F], UR, gs);
+  } else {
+    const int2* __restrict__ fx = reinterpret_cast<const int2*>(fq);
+    eval_side<2, false>(a.coef, a.cexp, a.hexp, a.N, o, fx[0], fx[F], fx[2 * F], UL, gs);
+    if (BND && nb < 0) ghost_state(-1 - nb, UL, n, a.uinf, UR);
+    else eval_side<2, true>(a.coef, a.cexp, a.hexp, a.N, nb, fx[3 * F], fx[4 * F], fx[5 * F], UR, gs);
+  }
   double flux[5];
   point_flux<VISC && !BND>(UL, UR, gs, n, VISC && !BND ? 2.0 * a.fpen[fc] : 0.0, a.c, flux);
 #pragma unroll
@@ -977,10 +1063,10 @@ __global__ void __launch_bounds__(kRedThreads) k_dt_fused(DtArgs a) {
 }
 
 // per-block sums [V KE, V |curl u|^2, V (div u)^2, V] in a fixed tree order, from
-// coefficients [K+1][N][5] (T = double: the FP64 form; float: the mixed form at P3/P4)
-template <typename T>
+// the FP64 form's coefficients [K+1][N][5] (in fixed point, of B bits, when cexp is given)
 __global__ void __launch_bounds__(kRedThreads)
-    k_diag_partial(const double* __restrict__ U, const T* __restrict__ coef, const double* __restrict__ vol, int N,
+    k_diag_partial(const double* __restrict__ U, const double* __restrict__ coef, const int32_t* __restrict__ cexp,
+                   const short4* __restrict__ hexp, int B, const double* __restrict__ vol, int N,
                    double* __restrict__ part) {
   __shared__ double sm[4][kRedThreads];
   double acc[4] = {0, 0, 0, 0};
@@ -989,10 +1075,23 @@ __global__ void __launch_bounds__(kRedThreads)
     const double r = U[i], ir = 1.0 / r;
     const double u[3] = {U[(size_t)N + i] * ir, U[2 * (size_t)N + i] * ir, U[3 * (size_t)N + i] * ir};
     double g[4][3];  // gradients of rho, m_x, m_y, m_z at the centroid (physical coefficients)
+    if (cexp) {
+      const short4 h = hexp[i];
+      const int hd[3] = {h.x, h.y, h.z};
 #pragma unroll
-    for (int v = 0; v < 4; v++)
+      for (int v = 0; v < 4; v++) {
+        const int e = cexp[(size_t)i * 5 + v] - B;
 #pragma unroll
-      for (int j = 0; j < 3; j++) g[v][j] = (double)coef[(j + 1) * st + (size_t)i * 5 + v];
+        for (int j = 0; j < 3; j++)
+          g[v][j] = fx_double(fx_value(*reinterpret_cast<const int2*>(coef + (j + 1) * st + (size_t)i * 5 + v)),
+                              e - hd[j]);
+      }
+    } else {
+#pragma unroll
+      for (int v = 0; v < 4; v++)
+#pragma unroll
+        for (int j = 0; j < 3; j++) g[v][j] = coef[(j + 1) * st + (size_t)i * 5 + v];
+    }
     double gu[3][3];
 #pragma unroll
     for (int q = 0; q < 3; q++)

@@ -44,7 +44,9 @@ struct ReconArgsHO {
   const double* __restrict__ Msi;   // [K(K+1)/2][N]: smoothness-indicator matrix, upper triangle by rows
   const double* __restrict__ psib;  // [K-3][N]: cell means of the basis monomials of degree >= 2
   const double* __restrict__ inv_h; // [N]
-  double* __restrict__ coef;        // [K+1][N][5] physical-unit monomial coefficients
+  const short4* __restrict__ hexp;  // [N] exponents of the cell's axis scales
+  double* __restrict__ coef;        // [K+1][N][5] physical-unit monomial coefficients, the non-constant ones in fixed point
+  int32_t* __restrict__ cexp;       // [N][5] their exponents
   int N;
   double lam0, lams, eps;
 };
@@ -155,63 +157,19 @@ __global__ void __launch_bounds__(128) k_recon_ho(ReconArgsHO a) {
   const size_t st = N * 5;
   out[0] = c0;
 #pragma unroll
-  for (int k = 0; k < K; k++) out[(k + 1) * st] = c[k] * ihp[basis_degree(k)];
+  for (int k = 0; k < K; k++) c[k] *= ihp[basis_degree(k)];
+  store_fixed<ORDER>(c, a.hexp[i], out, st, a.cexp + (size_t)i * 5 + v);
 }
 
-// value at the physical offset (x, y, z) from the centroid into U and the
-// gradient written (ACC = false) or added (ACC = true) into g
-template <int ORDER, bool ACC>
-__device__ __forceinline__ void eval_side_ho(const double* __restrict__ coef, int N, int cell, double x, double y,
-                                             double z, double U[5], double g[5][3]) {
-  constexpr int K = basis_count(ORDER);
-  const size_t st = (size_t)N * 5;
-  const double* p = coef + (size_t)cell * 5;
-  double px[ORDER + 1], py[ORDER + 1], pz[ORDER + 1];
-  px[0] = py[0] = pz[0] = 1.0;
-#pragma unroll
-  for (int e = 1; e <= ORDER; e++) {
-    px[e] = px[e - 1] * x;
-    py[e] = py[e - 1] * y;
-    pz[e] = pz[e - 1] * z;
-  }
-  double gx[5], gy[5], gz[5];
-#pragma unroll
-  for (int v = 0; v < 5; v++) {
-    U[v] = p[v];
-    gx[v] = gy[v] = gz[v] = 0.0;
-  }
-#pragma unroll
-  for (int k = 0; k < K; k++) {
-    const int ex = basis_exp(k, 0), ey = basis_exp(k, 1), ez = basis_exp(k, 2);
-    const double mv = px[ex] * py[ey] * pz[ez];
-    const double mx = ex ? ex * px[ex > 0 ? ex - 1 : 0] * py[ey] * pz[ez] : 0.0;
-    const double my = ey ? ey * px[ex] * py[ey > 0 ? ey - 1 : 0] * pz[ez] : 0.0;
-    const double mz = ez ? ez * px[ex] * py[ey] * pz[ez > 0 ? ez - 1 : 0] : 0.0;
-#pragma unroll
-    for (int v = 0; v < 5; v++) {
-      const double c = p[(k + 1) * st + v];
-      U[v] = fma(c, mv, U[v]);
-      if (ex) gx[v] = fma(c, mx, gx[v]);
-      if (ey) gy[v] = fma(c, my, gy[v]);
-      if (ez) gz[v] = fma(c, mz, gz[v]);
-    }
-  }
-#pragma unroll
-  for (int v = 0; v < 5; v++) {
-    if (ACC) {
-      g[v][0] += gx[v];
-      g[v][1] += gy[v];
-      g[v][2] += gz[v];
-    } else {
-      g[v][0] = gx[v];
-      g[v][1] = gy[v];
-      g[v][2] = gz[v];
-    }
-  }
-}
-
+// The point values and gradients are computed variable by variable in a loop that
+// stays rolled (its body is 1500 instructions at P4; unrolled over sides and
+// variables the kernel ran out of the instruction cache and of registers) and wait
+// in shared memory, one column per thread, for the flux.  Bound by the FP64 pipe and
+// its latency.  P4 at 24^3, us: evaluation in FP64 1635, in integers unrolled 969
+// (8 warps per SM), in this loop 548 (6, 8, 10 blocks per SM: 637, 548, 595).
+constexpr int kFaceHoThreads = 64;
 template <int ORDER, bool VISC>
-__global__ void __launch_bounds__(128) k_face_ho(FaceArgs a) {
+__global__ void __launch_bounds__(kFaceHoThreads, 8) k_face_ho(FaceArgs a) {
   constexpr int NQ = ORDER * ORDER, FPW = 32 / NQ;  // faces per warp
   const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   const int grp = lane / NQ, q = lane - NQ * (lane / NQ);
@@ -221,14 +179,37 @@ __global__ void __launch_bounds__(128) k_face_ho(FaceArgs a) {
   const int fc = live ? f : a.F - 1, qc = in_group ? q : 0;
   const size_t F = a.F;
   const double* __restrict__ fq = a.fq + (size_t)qc * 10 * F + fc;
-  const double xl = fq[0], yl = fq[F], zl = fq[2 * F];
-  const double xr = fq[3 * F], yr = fq[4 * F], zr = fq[5 * F];
+  const int2* __restrict__ fx = reinterpret_cast<const int2*>(fq);
   const double n[3] = {fq[6 * F], fq[7 * F], fq[8 * F]};
   const double area = fq[9 * F];
   const int o = a.fo[fc], nb = a.fn[fc];
-  double UL[5], UR[5], gs[5][3];  // gs = grad U_L + grad U_R
-  eval_side_ho<ORDER, false>(a.coef, a.N, o, xl, yl, zl, UL, gs);
-  eval_side_ho<ORDER, true>(a.coef, a.N, nb, xr, yr, zr, UR, gs);
+  __shared__ double sv[25][kFaceHoThreads];  // U_L, U_R, then grad U_L + grad U_R of each variable
+  const int t = threadIdx.x;
+  const size_t st = (size_t)a.N * 5;
+#pragma unroll 1
+  for (int side = 0; side < 2; side++) {
+    const int cell = side ? nb : o;
+    const int2* w = fx + (size_t)side * 3 * F;
+    const FxPoint<ORDER> pt(w[0], w[F], w[2 * F]);
+    const short4 h = __ldg(&a.hexp[cell]);
+    const double* p = a.coef + (size_t)cell * 5;
+#pragma unroll 1
+    for (int v = 0; v < 5; v++) {
+      double u, g[3];
+      pt.eval(p + v, st, a.cexp[(size_t)cell * 5 + v], h, u, g);
+      sv[side * 5 + v][t] = u;
+#pragma unroll
+      for (int d = 0; d < 3; d++) sv[10 + 3 * v + d][t] = side ? sv[10 + 3 * v + d][t] + g[d] : g[d];
+    }
+  }
+  double UL[5], UR[5], gs[5][3];
+#pragma unroll
+  for (int v = 0; v < 5; v++) {
+    UL[v] = sv[v][t];
+    UR[v] = sv[5 + v][t];
+#pragma unroll
+    for (int d = 0; d < 3; d++) gs[v][d] = sv[10 + 3 * v + d][t];
+  }
   double flux[5];
   point_flux<VISC>(UL, UR, gs, n, VISC ? 2.0 * a.fpen[fc] : 0.0, a.c, flux);
 #pragma unroll

@@ -63,11 +63,15 @@ struct DeviceMesh {
   int32_t* fo = nullptr;      // [F] owner
   int32_t* fn = nullptr;      // [F] neighbour; on a boundary face -1 - its boundary kind
   uint8_t* dvalid = nullptr;  // [N] bit s: directional candidate s exists (meshes with boundary faces)
-  double* fq = nullptr;       // [nq][10][F] x-x_L(3) x-x_R'(3) n(3) |dS|(1), physical offsets
+  double* fq = nullptr;       // [nq][10][F] x-x_L(3) x-x_R'(3) n(3) |dS|(1), physical offsets; FP64 form
+                              // from P2 on: offsets in fixed point (limb pairs), in units of their cell's axis scales
+  int16_t* hexp = nullptr;    // [N][4] exponents of the cell's axis scales (FP64 form from P2 on)
+  int32_t* cexp = nullptr;    // [N][5] exponents of the coefficients in fixed point (same)
   float* fqf = nullptr;       // FP32 copy, point-contiguous [F][nq][10]
   double* fpen = nullptr;     // [F] alpha / L_int
   // scratch owned by the handle
-  double* coef = nullptr;     // [NC][N][5] reconstructed monomial coefficients
+  double* coef = nullptr;     // [NC][N][5] reconstructed monomial coefficients (FP64 form from P2 on: from the
+                              // second on limb pairs in place of the doubles)
   float* coeff = nullptr;     // FP32 coefficients (mixed)
   float* Uhl = nullptr;       // [N][5][2] float pairs (hi, lo) of the state being reconstructed (mixed)
   double* G = nullptr;        // [5][F] face flux integrals (mixed form: [5][F] floats in the first half)

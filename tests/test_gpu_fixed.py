@@ -34,17 +34,32 @@ def _both(kind, n, order, scheme, Re=0.0, eps=1e-6, mach=0.5):
     return m, oc, I.noisy_state(nodes, cells, mach, 0.05, seed=6)
 
 
+# cells stretched 100:1 (10:1 at P4, where the oracle rejects the stencils beyond),
+# whose coefficients are scaled per axis
+@pytest.mark.parametrize("order,stretch", [(2, 100.0), (3, 100.0), (4, 10.0)])
+def test_stretched_cells(order, stretch):
+    nodes, cells, box = I.hex_lattice((10, 9, 9), length=(1.0, stretch, 3.0), jitter=0.1, seed=5)
+    p = dict(order=order, scheme=1, Re=1600.0, Mach=0.5)
+    m, oc = ucns.Mesh(nodes, cells, box, ucns.Params(**p)), O.Case(nodes, cells, box, O.Params(**p))
+    U = I.noisy_state(nodes, cells, 0.5, 0.05, seed=6)
+    R, (Rc, S) = _residual(m, U), oc.residual_terms(U)
+    err = np.abs(R - Rc).max(axis=1) / S.max(axis=1)
+    print(order, err)
+    assert np.all(err <= 1e-12)
+
+
 def _residual(m, U):
     R = m.residual(torch.from_numpy(np.ascontiguousarray(m.to_internal(U))).cuda())
     return m.to_user(R.cpu().numpy())
 
 
-# 210, 1050, 420, 1260 and 210 cells: the last 32-cell tile holds 18, 26, 4, 12 and 18;
+# 210, 1050, 420, 1260 and 210 cells: the last 32-cell tile holds 18, 26, 4, 12 and 18 (810 and
+# 900 at P3 and P4: 10 and 4);
 # eps 1e-60 with a uniform z momentum and states scaled by 2^200 leave the range in
 # which the weights share one denominator
 @pytest.mark.parametrize("kind,n,order,scheme", [
     ("hexes", (5, 6, 7), 2, 1), ("hexes", (5, 6, 7), 2, 0), ("tets", (5, 5, 7), 2, 1), ("prisms", (5, 6, 7), 2, 1),
-    ("pyramids", (5, 6, 7), 2, 1), ("walls", (5, 6, 7), 2, 1)])
+    ("pyramids", (5, 6, 7), 2, 1), ("walls", (5, 6, 7), 2, 1), ("hexes", (9, 9, 10), 3, 1), ("hexes", (9, 10, 10), 4, 1)])
 @pytest.mark.parametrize("eps,scale", [(1e-6, 0), (1e-60, 0), (1e-6, 200)])
 def test_residual_on_ragged_tiles(kind, n, order, scheme, eps, scale):
     m, oc, U = _both(kind, n, order, scheme, eps=eps)
@@ -60,14 +75,14 @@ def test_residual_on_ragged_tiles(kind, n, order, scheme, eps, scale):
 # The Euler residual with linear weights scales with the state; powers of two scale
 # exactly through every operation, also where the state lies below the range in
 # which differences are aligned directly (2^-962)
-@pytest.mark.parametrize("order", [2])
+@pytest.mark.parametrize("order", [2, 3, 4])
 @pytest.mark.parametrize("k", [-962, 600])
 def test_power_of_two_states_scale_exactly(order, k):
     m, _, U = _both("hexes", (9, 9, 10), order, 0, mach=1.0)
     assert np.array_equal(_residual(m, U * 2.0 ** k), _residual(m, U) * 2.0 ** k)
 
 
-@pytest.mark.parametrize("order", [2])
+@pytest.mark.parametrize("order", [2, 3, 4])
 @pytest.mark.parametrize("bad", [np.nan, np.inf])
 def test_non_finite_states_stay_visible(order, bad):
     m, oc, U = _both("hexes", (11, 11, 12), order, 0)
