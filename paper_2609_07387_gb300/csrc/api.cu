@@ -3,6 +3,7 @@
 // caller's stream.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <new>
@@ -73,16 +74,25 @@ int upload_blocked(T** dst, const std::vector<S>& src, int rows, int64_t N, bool
   return upload(dst, b);
 }
 
-// Rows k < K of cell i's least-squares matrix src [K][M][N] as limb pairs P and
-// exponents E, entry (k, m) at P[(k M + m) TC + c] (fixed.cuh)
-void fixed_rows(const double* src, int K, int M, int64_t N, int64_t i, int TC, int c, int2* P, int16_t* E) {
-  for (int k = 0; k < K; k++) {
-    double l1 = 0.0;
-    for (int m = 0; m < M; m++) l1 += std::fabs(src[((size_t)k * M + m) * N + i]);
-    const int e = fx_row_exponent(l1);
-    E[k * TC + c] = (int16_t)e;
-    const double up = std::ldexp(1.0, std::min(60 - e, 1000)), more = std::ldexp(1.0, std::max(60 - e - 1000, 0));
-    for (int m = 0; m < M; m++) P[(k * M + m) * TC + c] = fx_limbs(fx_round(src[((size_t)k * M + m) * N + i] * up * more));
+// One matrix row of nc <= 32 consecutive cells, entry m of cell c at row(m)[c], as
+// limb pairs at(m)[c] and exponents E[c] (fixed.cuh)
+template <class Row, class At>
+void fixed_row(const Row& row, int M, int nc, const At& at, int16_t* E) {
+  double l1[32] = {0.0}, up[32], more[32];
+  for (int m = 0; m < M; m++) {
+    const double* x = row(m);
+    for (int c = 0; c < nc; c++) l1[c] += std::fabs(x[c]);
+  }
+  for (int c = 0; c < nc; c++) {
+    const int e = fx_row_exponent(l1[c]);
+    E[c] = (int16_t)e;
+    up[c] = std::ldexp(1.0, std::min(60 - e, 1000));
+    more[c] = std::ldexp(1.0, std::max(60 - e - 1000, 0));
+  }
+  for (int m = 0; m < M; m++) {
+    const double* x = row(m);
+    int2* q = at(m);
+    for (int c = 0; c < nc; c++) q[c] = fx_limbs(fx_round(x[c] * up[c] * more[c]));
   }
 }
 
@@ -95,27 +105,85 @@ int upload_fx_tiles(const ucns_mesh* m, const HostArrays& h, unsigned char** dst
 #pragma omp parallel for schedule(static)
   for (int64_t t = 0; t < tiles; t++) {
     unsigned char* r = b.data() + (size_t)t * rec;
-    for (int c = 0; c < T::TC && t * T::TC + c < N; c++) {
-      const int64_t i = t * T::TC + c;
-      int32_t* id = reinterpret_cast<int32_t*>(r + T::C_ID);
-      for (int mm = 0; mm < T::MC; mm++) id[mm * T::TC + c] = h.sc[(size_t)mm * N + i];
-      fixed_rows(h.Pc.data(), T::K, T::MC, N, i, T::TC, c, reinterpret_cast<int2*>(r),
-                 reinterpret_cast<int16_t*>(r + T::C_EXP));
-      if (nd == 0) continue;
-      unsigned char* d = r + T::CENTRAL;
-      id = reinterpret_cast<int32_t*>(d + T::d_id(nd));
-      for (int mm = 0; mm < nd * T::MD; mm++) id[mm * T::TC + c] = h.sd[(size_t)mm * N + i];
-      fixed_rows(h.Pd.data(), nd * 3, T::MD, N, i, T::TC, c, reinterpret_cast<int2*>(d),
-                 reinterpret_cast<int16_t*>(d + T::d_exp(nd)));
-    }
+    const int64_t i0 = t * T::TC;
+    const int nc = (int)std::min<int64_t>(T::TC, N - i0);
+    auto rows = [&](const std::vector<double>& src, int K, int M, int2* P, int16_t* E) {
+      for (int k = 0; k < K; k++)
+        fixed_row([&](int mm) { return src.data() + ((size_t)k * M + mm) * N + i0; }, M, nc,
+                  [&](int mm) { return P + (k * M + mm) * T::TC; }, E + k * T::TC);
+    };
+    auto stencils = [&](const std::vector<int32_t>& src, int M, int32_t* id) {
+      for (int mm = 0; mm < M; mm++) std::copy_n(src.data() + (size_t)mm * N + i0, nc, id + mm * T::TC);
+    };
+    rows(h.Pc, T::K, T::MC, reinterpret_cast<int2*>(r), reinterpret_cast<int16_t*>(r + T::C_EXP));
+    stencils(h.sc, T::MC, reinterpret_cast<int32_t*>(r + T::C_ID));
+    if (nd == 0) continue;
+    unsigned char* dr = r + T::CENTRAL;
+    rows(h.Pd, nd * 3, T::MD, reinterpret_cast<int2*>(dr), reinterpret_cast<int16_t*>(dr + T::d_exp(nd)));
+    stencils(h.sd, nd * T::MD, reinterpret_cast<int32_t*>(dr + T::d_id(nd)));
   }
   return upload(dst, b);
 }
 
+// the P3/P4 reconstruction's tiles (HOFxTile) of the FP64 form, their stencils and row exponents
+template <int ORDER>
+int upload_ho_fx_tiles(const ucns_mesh* m, const HostArrays& h, DeviceMesh& d) {
+  using T = HOFxTile<ORDER>;
+  constexpr int K = T::K, MC = T::MC, KD = T::KD, MD = T::MD, TC = T::TC;
+  const bool weno = m->nd > 0;
+  const int64_t N = m->N, tiles = (N + TC - 1) / TC;
+  const int rec = T::record(weno);
+  std::vector<unsigned char> b((size_t)tiles * rec, 0);
+  std::vector<int32_t> ids((size_t)tiles * T::IDS * TC, 0);
+  std::vector<int16_t> exps((size_t)tiles * T::EXPS * TC, 0);
+#pragma omp parallel for schedule(static)
+  for (int64_t t = 0; t < tiles; t++) {
+    int2* r = reinterpret_cast<int2*>(b.data() + (size_t)t * rec);
+    int32_t* id = &ids[(size_t)t * T::IDS * TC];
+    int16_t* ex = &exps[(size_t)t * T::EXPS * TC];
+    const int64_t i0 = t * TC;
+    const int nc = (int)std::min<int64_t>(TC, N - i0);
+    for (int mm = 0; mm < MC; mm++) std::copy_n(h.sc.data() + (size_t)mm * N + i0, nc, id + mm * TC);
+    for (int k = 0; k < K; k++)
+      fixed_row([&](int mm) { return h.Pc.data() + ((size_t)k * MC + mm) * N + i0; }, MC, nc,
+                [&](int mm) {
+                  return r + (((k / 4) * T::NP + mm / T::MCH) * 4 * T::MCH + (k % 4) * T::MCH + mm % T::MCH) * TC;
+                },
+                ex + k * TC);
+    if (!weno) continue;
+    int2* at = r + T::CENTRAL / 8;
+    for (int g = 0; g < T::NG; g++) {
+      const int cols = K - 4 * g;  // columns from the group's first row on, in pieces of MCH
+      for (int rr = 0; rr < 4 && 4 * g + rr < K; rr++) {
+        const int k = 4 * g + rr;  // row k: zero below the diagonal, off-diagonal entries doubled
+        std::vector<double> x((size_t)cols * TC, 0.0);
+        for (int l = k; l < K; l++)
+          for (int c = 0; c < nc; c++)
+            x[(size_t)(l - 4 * g) * TC + c] =
+                (l == k ? 1.0 : 2.0) * h.Msi[(size_t)(k * K - k * (k - 1) / 2 + l - k) * N + i0 + c];
+        fixed_row([&](int l) { return x.data() + (size_t)l * TC; }, cols, nc,
+                  [&](int l) {
+                    const int p = l / T::MCH;
+                    return at + (4 * p * T::MCH + rr * T::si_columns(g, p) + l % T::MCH) * TC;
+                  },
+                  ex + (K + k) * TC);
+      }
+      at += 4 * cols * TC;
+    }
+    for (int mm = 0; mm < 6 * MD; mm++) std::copy_n(h.sd.data() + (size_t)mm * N + i0, nc, id + (MC + mm) * TC);
+    for (int k = 0; k < 6 * KD; k++)  // row k % KD of stencil k / KD
+      fixed_row([&](int mm) { return h.Pd.data() + ((size_t)k * MD + mm) * N + i0; }, MD, nc,
+                [&](int mm) { return at + ((k / 3) * 3 * MD + (k % 3) * MD + mm) * TC; }, ex + (2 * K + k) * TC);
+  }
+  int rc = upload(&d.fxt, b);
+  if (rc || (rc = upload(&d.fx_ids, ids))) return rc;
+  return upload(&d.fx_exps, exps);
+}
+
 // The FP64 face geometry from P2 on: per cell the exponents of its axis scales (the
 // powers of two above the largest |offset| of its face points along each axis),
-// and the offsets of fq as fixed-point limb pairs in those units
-int upload_fixed_faces(const ucns_mesh* m, double** dst, int16_t** dst_h, const std::vector<double>& fq) {
+// and the offsets of fq, in place, as fixed-point limb pairs in those units
+int upload_fixed_faces(const ucns_mesh* m, double** dst, int16_t** dst_h, std::vector<double>& fq) {
   const std::vector<int32_t>&fo = m->fo, &fn = m->fn;
   const int64_t F = m->F, N = m->N;
   const int nq = m->nq;
@@ -131,10 +199,9 @@ int upload_fixed_faces(const ucns_mesh* m, double** dst, int16_t** dst_h, const 
       }
       h[(size_t)i * 4 + d] = (int16_t)fx_row_exponent(big);
     }
-  std::vector<double> g(fq);
   for (int q = 0; q < nq; q++)
     for (int c = 0; c < 6; c++) {
-      double* row = &g[((size_t)q * 10 + c) * F];
+      double* row = &fq[((size_t)q * 10 + c) * F];
 #pragma omp parallel for schedule(static)
       for (int64_t f = 0; f < F; f++) {
         const int32_t i = c < 3 ? fo[f] : fn[f];
@@ -142,7 +209,7 @@ int upload_fixed_faces(const ucns_mesh* m, double** dst, int16_t** dst_h, const 
         std::memcpy(&row[f], &w, sizeof w);
       }
     }
-  int rc = upload(dst, g);
+  int rc = upload(dst, fq);
   return rc ? rc : upload(dst_h, h);
 }
 
@@ -404,35 +471,36 @@ int launch_face_mx(ucns_mesh* m, cudaStream_t s) {
 }
 
 // P3 / P4 (FP64, hexahedra)
+template <int ORDER, bool WENO>
+int launch_ho_fx_tiles(const ReconArgsHO& a, cudaStream_t s) {
+  using T = HOFxTile<ORDER>;
+  UCNS_CUDA(cudaFuncSetAttribute(k_recon_ho<ORDER, WENO>, cudaFuncAttributeMaxDynamicSharedMemorySize, T::SMEM));
+  k_recon_ho<ORDER, WENO><<<(unsigned)((a.N + T::TC - 1) / T::TC), T::THREADS, T::SMEM, s>>>(a);
+  UCNS_CUDA(cudaGetLastError());
+  return UCNS_OK;
+}
+
 int launch_recon_ho(ucns_mesh* m, const double* U, cudaStream_t s) {
   ReconArgsHO a;
   a.U = U;
-  a.sc = m->d.sc;
-  a.Pc = m->d.Pc;
-  a.sd = m->d.sd;
-  a.Pd = m->d.Pd;
+  a.tiles = m->d.fxt;
+  a.ids = m->d.fx_ids;
+  a.exps = m->d.fx_exps;
   a.Msi = m->d.Msi;
   a.psib = m->d.psib;
   a.inv_h = m->d.inv_h;
   a.hexp = reinterpret_cast<const short4*>(m->d.hexp);
   a.coef = m->d.coef;
   a.cexp = m->d.cexp;
+  a.err = m->d.err;
   a.N = (int)m->N;
   const double lsum = m->P.lambda_central + m->nd;
   a.lam0 = m->P.lambda_central / lsum;
   a.lams = 1.0 / lsum;
   a.eps = m->P.epsilon;
-  const unsigned g = nblocks((size_t)m->N * 5, 128);
   const bool weno = m->nd > 0;
-  if (m->K == 19) {
-    if (weno) k_recon_ho<3, true><<<g, 128, 0, s>>>(a);
-    else k_recon_ho<3, false><<<g, 128, 0, s>>>(a);
-  } else {
-    if (weno) k_recon_ho<4, true><<<g, 128, 0, s>>>(a);
-    else k_recon_ho<4, false><<<g, 128, 0, s>>>(a);
-  }
-  UCNS_CUDA(cudaGetLastError());
-  return UCNS_OK;
+  if (m->K == 19) return weno ? launch_ho_fx_tiles<3, true>(a, s) : launch_ho_fx_tiles<3, false>(a, s);
+  return weno ? launch_ho_fx_tiles<4, true>(a, s) : launch_ho_fx_tiles<4, false>(a, s);
 }
 
 int launch_face_ho(ucns_mesh* m, cudaStream_t s) {
@@ -960,7 +1028,7 @@ void device_free(ucns_mesh* m) {
   m->gate_eval_active = false;
   m->gate_fixed = false;
   DeviceMesh& d = m->d;
-  void* ptrs[] = {d.fslot, d.bcell, d.bcount, d.inv_vol, d.vol, d.inv_h, d.dtlen, d.mom, d.sc, d.Pc, d.sd, d.Pd, d.fxt, d.hexp, d.cexp, d.Msi, d.psib, d.hot, d.Msif, d.psibf, d.Pcb, d.Pdb, d.scb, d.sdb, d.cellb, d.sda, d.Pda,
+  void* ptrs[] = {d.fslot, d.bcell, d.bcount, d.inv_vol, d.vol, d.inv_h, d.dtlen, d.mom, d.sc, d.Pc, d.fxt, d.fx_ids, d.fx_exps, d.hexp, d.cexp, d.Msi, d.psib, d.hot, d.Msif, d.psibf, d.Pcb, d.Pdb, d.scb, d.sdb, d.cellb, d.sda, d.Pda,
                   d.inv_hf, d.fpenf, d.cf, d.fo, d.fn, d.dvalid, d.fq, d.fqf, d.fpen, d.coef, d.coeff, d.Uhl, d.G,
                   d.Ustage, d.Uacc, d.Uhost, d.red, d.dt, d.err, d.dt_part, d.dt_count};
   for (void* p : ptrs)
@@ -1132,7 +1200,7 @@ static void face_batches(const std::vector<int32_t>& fo, const std::vector<int32
 
 // the device arrays of a precomputed mesh (host vectors built here may
 // throw std::bad_alloc; the caller turns that into an error code)
-static int device_upload(ucns_mesh* m, const ucns_params* p, const HostArrays& h) {
+static int device_upload(ucns_mesh* m, const ucns_params* p, HostArrays& h) {
   int rc = UCNS_OK;
   device_free(m);
   m->precomputed = false;
@@ -1145,11 +1213,11 @@ static int device_upload(ucns_mesh* m, const ucns_params* p, const HostArrays& h
     for (int j = 0; j < m->nfc; j++) cf[(size_t)j * m->N + i] = m->cf[(size_t)i * m->nfc + j];
   for (int64_t f = 0; f < m->F; f++)
     if (fn[f] < 0) fn[f] = -1 - (int32_t)h.fkind[f];  // a boundary face carries its kind
-  // at P2 and in the mixed form the stencil ids lie in the reconstruction's tiles
-  const bool tiled = m->K == 9 || p->precision == UCNS_PREC_MIXED;
+  // from P2 on and in the mixed form the stencil ids lie in the reconstruction's tiles
+  const bool tiled = m->K >= 9 || p->precision == UCNS_PREC_MIXED;
   if ((rc = upload(&d.vol, h.vol)) || (rc = upload(&d.inv_vol, h.inv_vol)) ||
       (rc = upload(&d.inv_h, h.inv_h)) || (rc = upload(&d.dtlen, h.dtlen)) ||
-      (rc = upload(&d.mom, h.mom)) || (!tiled && ((rc = upload(&d.sc, h.sc)) || (rc = upload(&d.sd, h.sd)))) ||
+      (rc = upload(&d.mom, h.mom)) || (!tiled && (rc = upload(&d.sc, h.sc))) ||
       (rc = upload(&d.cf, cf)) || (rc = upload(&d.fo, fo)) || (rc = upload(&d.fn, fn)) ||
       (m->n_boundary > 0 && (rc = upload(&d.dvalid, h.dvalid)))) {
     device_free(m);
@@ -1196,7 +1264,8 @@ static int device_upload(ucns_mesh* m, const ucns_params* p, const HostArrays& h
       return rc;
     }
   } else if ((m->K == 9 && (rc = upload_fx_tiles(m, h, &d.fxt))) ||
-             (m->K != 9 && ((rc = upload(&d.Pc, h.Pc)) || (rc = upload(&d.Pd, h.Pd)))) ||
+             (m->K == 19 && (rc = upload_ho_fx_tiles<3>(m, h, d))) || (m->K == 34 && (rc = upload_ho_fx_tiles<4>(m, h, d))) ||
+             (m->K == 3 && (rc = upload(&d.Pc, h.Pc))) ||
              (m->K == 3 && (rc = upload(&d.fq, h.fq))) ||
              (m->K > 3 && ((rc = upload_fixed_faces(m, &d.fq, &d.hexp, h.fq)) ||
                             (rc = alloc(&d.cexp, (size_t)5 * m->N)))) ||

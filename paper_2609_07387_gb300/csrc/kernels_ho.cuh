@@ -1,14 +1,12 @@
 // P3 and P4 reconstruction and face kernels (FP64), hexahedra.
 //
-//   k_recon_ho  thread = (cell, variable): central least-squares contraction
-//               (K = 19 or 34 modes over 2K members, Eq. 4); with CWENOZ the
-//               six directional candidates (linear at P3, quadratic over 18
-//               members at P4, Sec. 2.2), the smoothness indicators as the
-//               quadratic forms a^T M a of each cell's precomputed matrix M
-//               (Eq. 6 reading), the nonlinear weights and the combination.
-//               The directional contractions run twice (once for the
-//               indicators, once for the combination) rather than holding all
-//               six candidates in registers.
+//   k_recon_ho  tile by tile, thread = (cell, variable): central least-squares
+//               contraction (K = 19 or 34 modes over 2K members, Eq. 4) in
+//               fixed point; with CWENOZ the six directional candidates
+//               (linear at P3, quadratic over 18 members at P4, Sec. 2.2), the
+//               smoothness indicators as the quadratic forms a^T M a of each
+//               cell's precomputed matrix M (Eq. 6 reading), the nonlinear
+//               weights and the combination.
 //   k_face_ho   ORDER^2 Gauss points per face on ORDER^2 lanes (9 at P3, 16
 //               at P4; 32 / ORDER^2 faces per warp); values and gradients of
 //               the monomial-form polynomials, HLLC, penalised viscous flux
@@ -35,18 +33,51 @@ struct HO {
   static constexpr int NQ = ORDER * ORDER;
 };
 
+// The FP64 form's reconstruction data, tile by tile (24 cells: four warps of (cell,
+// variable) threads, one on each scheduler), in fixed point (fixed.cuh).  Streamed
+// chunks: the central rows in groups of four, each in pieces of MCH members, [4][MCH][24]
+// limb pairs; with CWENOZ the smoothness matrix's rows in groups of four, upper
+// triangle (off-diagonal entries doubled), columns from the group's first row on in
+// pieces of MCH, [4][columns][24]; then per directional stencil its rows in groups of
+// three, [3][MD][24].  Rows past K and cells past N are zero.
+template <int ORDER>
+struct HOFxTile {
+  using H = HO<ORDER>;
+  static constexpr int K = H::K, MC = H::MC, KD = H::KD, MD = H::MD, TC = 24;
+  static constexpr int LANES = 128, THREADS = LANES + 32;  // 120 (cell, variable) threads and 8 spare ones, a copying warp
+  static constexpr int MCH = ORDER == 4 ? 17 : 19, NP = MC / MCH, NG = (K + 3) / 4, NGD = KD / 3;
+  static constexpr int CHUNK = 4 * MCH * TC * 8;  // bytes of a stage
+  static constexpr int DCHUNK = 3 * MD * TC * 8;
+  static constexpr int S = 3;
+  static constexpr int QB = MC * LANES * 8;  // operands of the sum at hand, one column per thread
+  // per tile: stencil ids [MC + 6 MD][24], row exponents [2 K + 6 KD][24] (central, matrix, directional)
+  static constexpr int IDS = MC + 6 * MD, EXPS = 2 * K + 6 * KD, EB = EXPS * TC * 2;
+  static constexpr int SMEM = QB + S * CHUNK + EB + 2 * S * 8 + 8;
+  UCNS_HD static constexpr int si_pieces(int g) { return (K - 4 * g + MCH - 1) / MCH; }
+  UCNS_HD static constexpr int si_columns(int g, int p) { return K - 4 * g - p * MCH < MCH ? K - 4 * g - p * MCH : MCH; }
+  // bytes of the smoothness matrix, and of a tile's record
+  UCNS_HD static constexpr int si_bytes() {
+    int n = 0;
+    for (int g = 0; g < NG; g++) n += 4 * (K - 4 * g) * TC * 8;
+    return n;
+  }
+  static constexpr int CENTRAL = NG * NP * CHUNK;
+  UCNS_HD static constexpr int record(bool weno) { return CENTRAL + (weno ? si_bytes() + 6 * NGD * DCHUNK : 0); }
+  static_assert(MC % MCH == 0 && EB % 16 == 0 && 6 * KD <= MC && DCHUNK <= CHUNK && CHUNK % 16 == 0 && DCHUNK % 16 == 0 && QB % 16 == 0, "whole chunks");
+};
+
 struct ReconArgsHO {
   const double* __restrict__ U;     // [5][N]
-  const int32_t* __restrict__ sc;   // [MC][N]
-  const double* __restrict__ Pc;    // [K][MC][N]
-  const int32_t* __restrict__ sd;   // [6][MD][N]
-  const double* __restrict__ Pd;    // [6][KD][MD][N]
+  const unsigned char* __restrict__ tiles;  // records (HOFxTile)
+  const int32_t* __restrict__ ids;          // [tiles][IDS][24]
+  const int16_t* __restrict__ exps;         // [tiles][EXPS][24]
   const double* __restrict__ Msi;   // [K(K+1)/2][N]: smoothness-indicator matrix, upper triangle by rows
   const double* __restrict__ psib;  // [K-3][N]: cell means of the basis monomials of degree >= 2
   const double* __restrict__ inv_h; // [N]
   const short4* __restrict__ hexp;  // [N] exponents of the cell's axis scales
   double* __restrict__ coef;        // [K+1][N][5] physical-unit monomial coefficients, the non-constant ones in fixed point
   int32_t* __restrict__ cexp;       // [N][5] their exponents
+  int* err;                         // bit 1: a copy wait gave up
   int N;
   double lam0, lams, eps;
 };
@@ -67,55 +98,218 @@ __device__ __forceinline__ double si_form(const double* __restrict__ M, size_t N
   return s;
 }
 
-// directional candidate s of variable v: b = P_s (U_m - U_i) over its members
-template <int ORDER>
-__device__ __forceinline__ void dir_coeffs(const ReconArgsHO& a, const double* __restrict__ Uv, double ui, int i, int s,
-                                           double (&b)[HO<ORDER>::KD]) {
-  using H = HO<ORDER>;
-  const size_t N = a.N;
-#pragma unroll
-  for (int k = 0; k < H::KD; k++) b[k] = 0.0;
-#pragma unroll 2
-  for (int r = 0; r < H::MD; r++) {
-    const int j = __ldg(&a.sd[((size_t)s * H::MD + r) * N + i]);
-    const double d = Uv[j] - ui;
-#pragma unroll
-    for (int k = 0; k < H::KD; k++) b[k] = fma(__ldg(&a.Pd[(((size_t)s * H::KD + k) * H::MD + r) * N + i]), d, b[k]);
-  }
-}
-
+// One block per 24-cell tile: thread (cell c, variable v) = 5 c + v, plus a copying
+// warp that streams the tile's chunks through a ring of S shared-memory stages, every
+// wait bounded.  The differences of a stencil wait in shared memory as operands while
+// its rows pass; the central coefficients (xi units) wait in the output array.
+// Bound by latency at two warps per scheduler (issue 30 %, FP64 pipe 25 %): 11
+// thousand integer multiply-adds a thread at P4.  P4 CWENOZ at 24^3, us: FP64
+// contractions from global memory 852, this 339 (418 with the directional
+// contractions run twice and the row exponents read from global memory).
 template <int ORDER, bool WENO>
-__global__ void __launch_bounds__(128) k_recon_ho(ReconArgsHO a) {
-  using H = HO<ORDER>;
-  constexpr int K = H::K, MC = H::MC, KD = H::KD, ND = 6;
-  const int tid = blockIdx.x * blockDim.x + threadIdx.x;
-  const int i = tid / 5, v = tid - 5 * (tid / 5);
-  if (i >= a.N) return;
+__global__ void __launch_bounds__(HOFxTile<ORDER>::THREADS, 2) k_recon_ho(ReconArgsHO a) {
+  using T = HOFxTile<ORDER>;
+  constexpr int K = T::K, MC = T::MC, KD = T::KD, MD = T::MD, ND = 6, TC = T::TC, S = T::S, L = T::LANES;
+  extern __shared__ __align__(128) unsigned char smem[];
+  long long* sQ = reinterpret_cast<long long*>(smem);
+  unsigned char* ring = smem + T::QB;
+  unsigned char* sE = ring + S * T::CHUNK;  // the row exponents
+  uint64_t* full = reinterpret_cast<uint64_t*>(sE + T::EB);
+  uint64_t* empty = full + S;
+  uint64_t* ebar = empty + S;
+  const int t = threadIdx.x, lane = t & 31, tile = blockIdx.x;
+  if (t < S) {
+    bar_init(&full[t]);
+    bar_init(&empty[t], L / 32);
+  }
+  if (t == S) bar_init(ebar);
+  __syncthreads();
+  if (t >= L) {  // the copying warp
+    if (lane != 0) return;
+    bar_expect(ebar, T::EB);
+    bulk_load(sE, a.exps + (size_t)tile * T::EXPS * TC, T::EB, ebar);
+    const unsigned char* rec = a.tiles + (size_t)tile * T::record(WENO);
+    int q = 0;
+    bool ok = true;
+    auto put = [&](const unsigned char* src, int bytes) {
+      ok = ok && (q < S || bar_wait(&empty[q % S], (uint32_t)(q / S + 1) & 1u));
+      if (!ok) return;
+      bar_expect(&full[q % S], (uint32_t)bytes);
+      bulk_load(ring + (q % S) * T::CHUNK, src, (uint32_t)bytes, &full[q % S]);
+      q++;
+    };
+    for (int n = 0; n < T::NG * T::NP && ok; n++) put(rec + (size_t)n * T::CHUNK, T::CHUNK);
+    if constexpr (WENO) {
+      const unsigned char* src = rec + T::CENTRAL;
+      for (int g = 0; g < T::NG; g++)
+        for (int p = 0; p < T::si_pieces(g) && ok; p++) {
+          const int bytes = 4 * T::si_columns(g, p) * TC * 8;
+          put(src, bytes);
+          src += bytes;
+        }
+      for (int n = 0; n < ND * T::NGD && ok; n++) put(src + (size_t)n * T::DCHUNK, T::DCHUNK);
+    }
+    if (!ok) atomicOr(a.err, 2);
+    bar_wait(ebar, 0);
+    // the last copies into each stage land before the block's shared memory is released
+    for (int n = q - 1; n >= 0 && n >= q - S; n--) bar_wait(&full[n % S], (uint32_t)(n / S) & 1u);
+    return;
+  }
+  const int c = t < 5 * TC ? t / 5 : 0, v = t < 5 * TC ? t - 5 * c : 0;
+  const bool live = t < 5 * TC && tile * TC + c < a.N;
+  const int i = min(tile * TC + c, a.N - 1);
   const size_t N = a.N;
   const double* __restrict__ Uv = a.U + (size_t)v * N;
   const double ui = Uv[i];
-  double ao[K];
-#pragma unroll
-  for (int k = 0; k < K; k++) ao[k] = 0.0;
-#pragma unroll 2
-  for (int m = 0; m < MC; m++) {
-    const int j = __ldg(&a.sc[(size_t)m * N + i]);
-    const double d = Uv[j] - ui;
-#pragma unroll
-    for (int k = 0; k < K; k++) ao[k] = fma(__ldg(&a.Pc[((size_t)k * MC + m) * N + i]), d, ao[k]);
+  const int32_t* __restrict__ ids = a.ids + (size_t)tile * T::IDS * TC + c;
+  const int16_t* exps = reinterpret_cast<const int16_t*>(sE) + c;
+  double* out = a.coef + (size_t)i * 5 + v;
+  const size_t st = N * 5;
+  int q = 0;
+  bool ok = __all_sync(0xffffffffu, bar_wait(ebar, 0));
+  auto take = [&]() {  // wait for chunk q
+    ok = ok && __all_sync(0xffffffffu, bar_wait(&full[q % S], (uint32_t)(q / S) & 1u));
+    return reinterpret_cast<const int2*>(ring + (q % S) * T::CHUNK) + c;
+  };
+  auto give = [&]() {  // this warp is done with chunk q
+    __syncwarp();
+    if (lane == 0) bar_arrive(&empty[q % S]);
+    q++;
+  };
+  // the differences of the central stencil as operands (fx_differences, by way of shared memory)
+  constexpr int B = fx_bits_of(MC);
+  int ec;
+  {
+    long long* col = sQ + t;
+    int eb = fx_exponent(ui);
+#pragma unroll 17
+    for (int m = 0; m < MC; m++) {
+      const double u = Uv[ids[m * TC]];
+      col[m * L] = __double_as_longlong(u);
+      eb = max(eb, fx_exponent(u));
+    }
+    const bool low = eb < 64;
+    const double up = low ? 0x1p512 : 1.0;
+    if (low) {
+      eb = fx_exponent(ui * up);
+      for (int m = 0; m < MC; m++) {
+        const double u = __longlong_as_double(col[m * L]) * up;
+        col[m * L] = __double_as_longlong(u);
+        eb = max(eb, fx_exponent(u));
+      }
+    }
+    const long long f0 = fx_integer(low ? ui * up : ui, eb);
+    unsigned long long any = 1;
+#pragma unroll 4
+    for (int m = 0; m < MC; m++) {
+      const long long d = fx_integer(__longlong_as_double(col[m * L]), eb) - f0;
+      col[m * L] = d;
+      any |= (unsigned long long)(d ^ (d >> 63));
+    }
+    const int lz = fx_clz(any);
+#pragma unroll 4
+    for (int m = 0; m < MC; m++) {
+      const int2 w = fx_limbs(((col[m * L] << (lz - 1)) + (1ll << (62 - B))) >> (63 - B));
+      *reinterpret_cast<int2*>(&col[m * L]) = w;
+    }
+    ec = eb == 2047 ? kFxNan : eb - 1020 - lz - (low ? 512 : 0);
   }
-  double c[K];
-  if constexpr (!WENO) {
+  const int2* op = reinterpret_cast<const int2*>(sQ) + t;
+  int ea = 0;  // largest biased exponent of the central coefficients
+#pragma unroll 1
+  for (int g = 0; g < T::NG; g++) {
+    FxAcc acc[4];
+#pragma unroll 1
+    for (int p = 0; p < T::NP; p++) {
+      const int2* ch = take();
+      if (!ok) break;
 #pragma unroll
-    for (int k = 0; k < K; k++) c[k] = ao[k];
-  } else {
-    const double SI0 = si_form<K, K>(a.Msi, N, i, ao);
+      for (int m = 0; m < T::MCH; m++) {
+        const int2 w = op[(p * T::MCH + m) * L];
+#pragma unroll
+        for (int r = 0; r < 4; r++) fx_mac(acc[r], ch[(r * T::MCH + m) * TC], w);
+      }
+      give();
+    }
+    if (!ok) break;
+#pragma unroll
+    for (int r = 0; r < 4; r++)
+      if (4 * g + r < K) {
+        const double x = fx_double(fx_sum(acc[r]), (int)exps[(4 * g + r) * TC] + ec - 2 - B);
+        ea = max(ea, fx_exponent(x));
+        if (live) out[(4 * g + r + 1) * st] = x;
+      }
+  }
+  double r0 = 1.0;
+  double cd[KD];  // the leading modes' part of the directional candidates
+#pragma unroll
+  for (int k = 0; k < KD; k++) cd[k] = 0.0;
+  if constexpr (WENO) {
+    // a^T M a of the central coefficients, rows t_k = sum_{l >= k} M_kl a_l in integers
+    // (coefficients below 2^-959 have no square in FP64: the sum is zero)
+    constexpr int BA = fx_bits_of(K);
+#pragma unroll
+    for (int k = 0; k < K; k++)
+      *reinterpret_cast<int2*>(&sQ[k * L + t]) = fx_operand<BA>(live ? out[(k + 1) * st] : 0.0, ea);
+    const int es = ea == 2047 ? kFxNan : ea - 1022;
+    double SI0 = 0.0;
+#pragma unroll 1
+    for (int g = 0; g < T::NG && ok; g++) {
+      FxAcc acc[4];
+      double ak[4];
+#pragma unroll
+      for (int r = 0; r < 4; r++) ak[r] = 4 * g + r < K && live ? out[(4 * g + r + 1) * st] : 0.0;
+#pragma unroll 1
+      for (int p = 0; p < T::si_pieces(g); p++) {
+        const int2* ch = take();
+        if (!ok) break;
+        const int nc = T::si_columns(g, p);
+#pragma unroll 4
+        for (int m = 0; m < nc; m++) {
+          const int2 w = op[(4 * g + p * T::MCH + m) * L];
+#pragma unroll
+          for (int r = 0; r < 4; r++) fx_mac(acc[r], ch[(r * nc + m) * TC], w);
+        }
+        give();
+      }
+#pragma unroll
+      for (int r = 0; r < 4; r++)
+        if (4 * g + r < K && ea >= 64)
+          SI0 = fma(ak[r], fx_double(fx_sum(acc[r]), (int)exps[(K + 4 * g + r) * TC] + es - 2 - BA), SI0);
+    }
+    // directional candidate s: b = P_s (U_m - U_i) over its members
+    constexpr int BD = fx_bits_of(MD);
+    auto candidate = [&](int s, double (&b)[KD]) {
+      double u[MD];
+#pragma unroll
+      for (int m = 0; m < MD; m++) u[m] = Uv[ids[(MC + s * MD + m) * TC]];
+      int2 w[MD];
+      int e;
+      fx_differences<MD>(u, ui, w, e);
+#pragma unroll
+      for (int g = 0; g < T::NGD; g++) {
+        const int2* ch = take();
+        if (!ok) return;
+#pragma unroll
+        for (int r = 0; r < 3; r++) {
+          FxAcc acc;
+#pragma unroll
+          for (int m = 0; m < MD; m++) fx_mac(acc, ch[(r * MD + m) * TC], w[m]);
+          b[3 * g + r] = fx_double(fx_sum(acc), (int)exps[(2 * K + s * KD + 3 * g + r) * TC] + e - 2 - BD);
+        }
+        give();
+      }
+    };
     double SI[ND];
     double tau = 0.0;
+    double* sB = reinterpret_cast<double*>(sQ) + t;  // the candidates wait where the operands were
 #pragma unroll 1
-    for (int s = 0; s < ND; s++) {
+    for (int s = 0; s < ND && ok; s++) {
       double b[KD];
-      dir_coeffs<ORDER>(a, Uv, ui, i, s, b);
+      candidate(s, b);
+      if (!ok) break;
+#pragma unroll
+      for (int k = 0; k < KD; k++) sB[(s * KD + k) * L] = b[k];
       SI[s] = si_form<K, KD>(a.Msi, N, i, b);
       tau += fabs(SI0 - SI[s]);
     }
@@ -131,34 +325,39 @@ __global__ void __launch_bounds__(128) k_recon_ho(ReconArgsHO a) {
     }
     const double iws = 1.0 / wsum;
     // p = omega_0 p_1 + sum_s omega_s p_s with p_1 = (p_opt - sum lambda_s p_s)/lambda_0
-    const double r0 = (w0 * iws) / a.lam0;
+    r0 = (w0 * iws) / a.lam0;
 #pragma unroll
-    for (int k = 0; k < K; k++) c[k] = r0 * ao[k];
-#pragma unroll 1
     for (int s = 0; s < ND; s++) {
-      double b[KD];
-      dir_coeffs<ORDER>(a, Uv, ui, i, s, b);
       const double e = ws[s] * iws - r0 * a.lams;
 #pragma unroll
-      for (int k = 0; k < KD; k++) c[k] = fma(e, b[k], c[k]);
+      for (int k = 0; k < KD; k++) cd[k] = fma(e, sB[(s * KD + k) * L], cd[k]);
     }
+  }
+  if (!ok) {
+    if (lane == 0) atomicOr(a.err, 2);
+    return;
+  }
+  if (!live) return;
+  double cf[K];
+#pragma unroll
+  for (int k = 0; k < K; k++) {
+    const double ao = out[(k + 1) * st];
+    cf[k] = WENO ? fma(r0, ao, k < KD ? cd[k < KD ? k : 0] : 0.0) : ao;
   }
   // monomial form in physical units: p = c0 + sum_k (c_k / h^deg_k) (x - x_i)^e_k,
   // c0 = U_i - sum_{deg >= 2} c_k mean(psi_k)
   double c0 = ui;
 #pragma unroll
-  for (int k = 3; k < K; k++) c0 = fma(-c[k], __ldg(&a.psib[(size_t)(k - 3) * N + i]), c0);
+  for (int k = 3; k < K; k++) c0 = fma(-cf[k], __ldg(&a.psib[(size_t)(k - 3) * N + i]), c0);
   const double ih = __ldg(&a.inv_h[i]);
   double ihp[ORDER + 1];
   ihp[0] = 1.0;
 #pragma unroll
   for (int e = 1; e <= ORDER; e++) ihp[e] = ihp[e - 1] * ih;
-  double* out = a.coef + (size_t)i * 5 + v;
-  const size_t st = N * 5;
   out[0] = c0;
 #pragma unroll
-  for (int k = 0; k < K; k++) c[k] *= ihp[basis_degree(k)];
-  store_fixed<ORDER>(c, a.hexp[i], out, st, a.cexp + (size_t)i * 5 + v);
+  for (int k = 0; k < K; k++) cf[k] *= ihp[basis_degree(k)];
+  store_fixed<ORDER>(cf, a.hexp[i], out, st, a.cexp + (size_t)i * 5 + v);
 }
 
 // The point values and gradients are computed variable by variable in a loop that

@@ -32,11 +32,11 @@ struct DeviceMesh {
   double* inv_h = nullptr;    // [N] 1/h_i, h_i = V_i^(1/3)
   double* dtlen = nullptr;    // [N] CFL length 2 V_i / sum_f |S_f|
   double* mom = nullptr;      // [6][N] (1/V) int xi_a xi_b: xx yy zz xy xz yz
-  int32_t* sc = nullptr;      // [Mc][N] central stencil
-  double* Pc = nullptr;       // [K][Mc][N] central pseudo-inverse
-  int32_t* sd = nullptr;      // [nd][Md][N] directional stencils
-  double* Pd = nullptr;       // [nd][Kd][Md][N]
-  unsigned char* fxt = nullptr;  // FP64 form at P2: stencils and least-squares rows in fixed point, 32-cell tiles
+  int32_t* sc = nullptr;      // [6][N] central stencil (FP64 form at P1)
+  double* Pc = nullptr;       // [3][6][N] central pseudo-inverse (FP64 form at P1)
+  unsigned char* fxt = nullptr;  // FP64 form from P2 on: least-squares rows in fixed point, tile by tile (P2: and stencils)
+  int32_t* fx_ids = nullptr;     // FP64 form at P3/P4: [tiles][IDS][24] stencils
+  int16_t* fx_exps = nullptr;    // [tiles][EXPS][24] row exponents
   double* Msi = nullptr;      // P3/P4: [K(K+1)/2][N] smoothness-indicator matrix (upper triangle, row-major)
   float* hot = nullptr;       // P3/P4 mixed form: stencil ids and FP32 pseudo-inverses in 64-cell tiles; FP32 Msi, psib
   float* Msif = nullptr;
