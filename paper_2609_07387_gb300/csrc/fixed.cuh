@@ -135,7 +135,8 @@ __host__ __device__ __forceinline__ long long fx_integer(double x, int eb) {
   const unsigned long long b = fx_bits(x);
   const int e = (int)((unsigned)(b >> 52) & 0x7ffu);
   const unsigned long long mant = (b & 0xfffffffffffffull) | ((unsigned long long)(e != 0) << 52);
-  const unsigned long long q = (mant << 9) >> (eb - e < 63 ? eb - e : 63);
+  const int sh = eb - (e > 1 ? e : 1);
+  const unsigned long long q = (mant << 9) >> (sh < 63 ? sh : 63);
   const unsigned long long sgn = (unsigned long long)((long long)b >> 63);
   return (long long)((q ^ sgn) - sgn);
 }
@@ -229,5 +230,27 @@ __host__ __device__ __forceinline__ int2 fx_mul(int2 a, int2 b) {
 
 // the integer hi 2^30 + lo
 __host__ __device__ __forceinline__ long long fx_value(int2 q) { return ((long long)q.x << 30) + q.y; }
+
+// a number s 2^e, |s| <= 2^62.2
+struct FxSum {
+  long long s;
+  int e;
+};
+
+__host__ __device__ __forceinline__ FxSum fx_of(double x) {
+  const int eb = fx_exponent(x);
+  return {fx_integer(x, eb > 1 ? eb : 1), eb == 2047 ? kFxNan : (eb > 1 ? eb : 1) - 1084};
+}
+
+// a + b, the one of the smaller unit shifted to the larger (61 bits of the larger
+// kept): rounded to FP64 afterwards, closer than FP64 terms added
+__host__ __device__ __forceinline__ FxSum fx_add(FxSum a, FxSum b) {
+  const bool swap = a.e < b.e;
+  const FxSum x = swap ? b : a, y = swap ? a : b;
+  const int d = x.e - y.e < 62 ? x.e - y.e : 62;
+  return {(x.s >> 1) + (y.s >> (d + 1)), x.e + 1};
+}
+
+__host__ __device__ __forceinline__ double fx_double(FxSum a) { return fx_double(a.s, a.e); }
 
 }  // namespace ucns

@@ -510,8 +510,9 @@ __device__ __forceinline__ void eval_side_p1(const double* __restrict__ coef, in
 // From P2 on: the same at the offset (x, y, z), fixed point in units of the cell's
 // axis scales: products and sums on the integer pipe (fixed.cuh), one rounding to
 // FP64 of each value and gradient component.  k_face<2> at 72 x 80 x 88, us: FP64
-// evaluation 4756 (165 of its 430 FP64 operations a point), this 3220 (the FP64 pipe
-// busy 85 %).
+// evaluation 4756 (165 of its 430 FP64 operations a point), integer sums 3220 (the FP64
+// pipe busy 85 %), the constant term and the two gradients added as integers too 2974
+// (at 6, 8, 10 blocks per SM 3059, 2974, 3024).
 template <int ORDER>
 struct FxPoint {
   int2 m[basis_count(ORDER)];  // the monomials
@@ -527,7 +528,7 @@ struct FxPoint {
   }
   // value u and gradient g of one variable: p its constant term (the others st
   // doubles apart each), e its exponent, h the cell's axis scales
-  __device__ __forceinline__ void eval(const double* p, size_t st, int e, short4 h, double& u, double (&g)[3]) const {
+  __device__ __forceinline__ void eval(const double* p, size_t st, int e, short4 h, double& u, FxSum (&g)[3]) const {
     FxAcc a, s[3];
     long long lin[3];
 #pragma unroll
@@ -549,27 +550,30 @@ struct FxPoint {
       }
     }
     e -= fx_coef_bits(ORDER);
-    u = *p + fx_double(fx_sum(a), e);
+    u = fx_double(fx_add(fx_of(*p), {fx_sum(a), e}));
     const int hd[3] = {h.x, h.y, h.z};
 #pragma unroll
-    for (int d = 0; d < 3; d++) g[d] = fx_double(fx_sum(s[d]) + lin[d], e - hd[d]);
+    for (int d = 0; d < 3; d++) g[d] = {fx_sum(s[d]) + lin[d], e - hd[d]};
   }
 };
 
-template <int ORDER, bool ACC>
-__device__ __forceinline__ void eval_side(const double* __restrict__ coef, const int32_t* __restrict__ cexp,
-                                          const short4* __restrict__ hexp, int N, int cell, int2 x, int2 y, int2 z,
-                                          double U[5], double g[5][3]) {
-  const size_t st = (size_t)N * 5;
-  const double* p = coef + (size_t)cell * 5;
-  const short4 h = __ldg(&hexp[cell]);
-  const FxPoint<ORDER> pt(x, y, z);
+// both sides' values and the sum of their gradients; nb < 0: the owner's values and gradients alone
+template <int ORDER>
+__device__ __forceinline__ void eval_sides(const FaceArgs& a, int o, int nb, const int2* __restrict__ fx, size_t F,
+                                           double UL[5], double UR[5], double gs[5][3]) {
+  const size_t st = (size_t)a.N * 5;
+  const FxPoint<ORDER> pl(fx[0], fx[F], fx[2 * F]);
+  const short4 hl = __ldg(&a.hexp[o]);
+  const int n = nb < 0 ? o : nb;
+  const FxPoint<ORDER> pr(fx[3 * F], fx[4 * F], fx[5 * F]);
+  const short4 hr = __ldg(&a.hexp[n]);
 #pragma unroll
   for (int v = 0; v < 5; v++) {
-    double t[3];
-    pt.eval(p + v, st, cexp[(size_t)cell * 5 + v], h, U[v], t);
+    FxSum gl[3], gr[3];
+    pl.eval(a.coef + (size_t)o * 5 + v, st, a.cexp[(size_t)o * 5 + v], hl, UL[v], gl);
+    pr.eval(a.coef + (size_t)n * 5 + v, st, a.cexp[(size_t)n * 5 + v], hr, UR[v], gr);
 #pragma unroll
-    for (int d = 0; d < 3; d++) g[v][d] = ACC ? g[v][d] + t[d] : t[d];
+    for (int d = 0; d < 3; d++) gs[v][d] = fx_double(fx_add(gl[d], gr[d]));
   }
 }
 
@@ -598,7 +602,7 @@ __device__ __forceinline__ void ghost_state(int kind, const double UL[5], const 
 // mesh has boundary faces (neighbour id -1 - kind), whose flux is HLLC
 // between the owner's state and its ghost state (inviscid flows only)
 template <int ORDER, bool VISC, bool BND = false>
-__global__ void __launch_bounds__(256) k_face(FaceArgs a) {
+__global__ void __launch_bounds__(64, 8) k_face(FaceArgs a) {
   constexpr int NQ = ORDER * ORDER;
   const int tid = blockIdx.x * blockDim.x + threadIdx.x;
   const int f = tid / NQ, q = tid - NQ * (tid / NQ);
@@ -615,10 +619,8 @@ __global__ void __launch_bounds__(256) k_face(FaceArgs a) {
     if (BND && nb < 0) ghost_state(-1 - nb, UL, n, a.uinf, UR);
     else eval_side_p1<true>(a.coef, a.N, nb, fq[3 * F], fq[4 * F], fq[5 * F], UR, gs);
   } else {
-    const int2* __restrict__ fx = reinterpret_cast<const int2*>(fq);
-    eval_side<2, false>(a.coef, a.cexp, a.hexp, a.N, o, fx[0], fx[F], fx[2 * F], UL, gs);
+    eval_sides<2>(a, o, nb, reinterpret_cast<const int2*>(fq), F, UL, UR, gs);
     if (BND && nb < 0) ghost_state(-1 - nb, UL, n, a.uinf, UR);
-    else eval_side<2, true>(a.coef, a.cexp, a.hexp, a.N, nb, fx[3 * F], fx[4 * F], fx[5 * F], UR, gs);
   }
   double flux[5];
   point_flux<VISC && !BND>(UL, UR, gs, n, VISC && !BND ? 2.0 * a.fpen[fc] : 0.0, a.c, flux);

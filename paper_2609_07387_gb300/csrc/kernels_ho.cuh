@@ -365,7 +365,8 @@ __global__ void __launch_bounds__(HOFxTile<ORDER>::THREADS, 2) k_recon_ho(ReconA
 // variables the kernel ran out of the instruction cache and of registers) and wait
 // in shared memory, one column per thread, for the flux.  Bound by the FP64 pipe and
 // its latency.  P4 at 24^3, us: evaluation in FP64 1635, in integers unrolled 969
-// (8 warps per SM), in this loop 548 (6, 8, 10 blocks per SM: 637, 548, 595).
+// (8 warps per SM), in this loop 548 (6, 8, 10 blocks per SM: 637, 548, 595), the
+// constant term added as an integer 534.
 constexpr int kFaceHoThreads = 64;
 template <int ORDER, bool VISC>
 __global__ void __launch_bounds__(kFaceHoThreads, 8) k_face_ho(FaceArgs a) {
@@ -394,11 +395,15 @@ __global__ void __launch_bounds__(kFaceHoThreads, 8) k_face_ho(FaceArgs a) {
     const double* p = a.coef + (size_t)cell * 5;
 #pragma unroll 1
     for (int v = 0; v < 5; v++) {
-      double u, g[3];
+      double u;
+      FxSum g[3];
       pt.eval(p + v, st, a.cexp[(size_t)cell * 5 + v], h, u, g);
       sv[side * 5 + v][t] = u;
 #pragma unroll
-      for (int d = 0; d < 3; d++) sv[10 + 3 * v + d][t] = side ? sv[10 + 3 * v + d][t] + g[d] : g[d];
+      for (int d = 0; d < 3; d++) {
+        const double x = fx_double(g[d]);
+        sv[10 + 3 * v + d][t] = side ? sv[10 + 3 * v + d][t] + x : x;
+      }
     }
   }
   double UL[5], UR[5], gs[5][3];
