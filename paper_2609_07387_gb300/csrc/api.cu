@@ -297,6 +297,13 @@ FluxConstF flux_const_f(const ucns_params& p) {
 
 bool mixed(const ucns_mesh* m) { return m->P.precision == UCNS_PREC_MIXED; }
 
+// entries of the linear terms in a mixed-form coefficient row
+int3 linear_entries(const ucns_mesh* m) {
+  if (m->K <= 9) return make_int3(1, 2, 3);
+  const int r = m->K == 19 ? 3 : 4;
+  return make_int3(horner_place(0, r), horner_place(1, r), horner_place(2, r));
+}
+
 // floats per cell row of the mixed-form coefficients: 5 (K+1) rounded up to 4
 int coef_row_floats(const ucns_mesh* m) { return (5 * m->NC + 3) / 4 * 4; }
 
@@ -863,7 +870,7 @@ void launch_diag_partial(ucns_mesh* m, const double* U, cudaStream_t s) {
 // the last reconstruction left, into out[0..3] (device)
 int diag_sums_into(ucns_mesh* m, const double* U, double* out, cudaStream_t s) {
   if (mixed(m))
-    k_diag_partial_mx<<<m->d.red_blocks, kRedThreads, 0, s>>>(U, m->d.coeff, coef_row_floats(m), m->NC, m->d.vol,
+    k_diag_partial_mx<<<m->d.red_blocks, kRedThreads, 0, s>>>(U, m->d.coeff, coef_row_floats(m), m->NC, linear_entries(m), m->d.vol,
                                                              (int)m->N, m->d.red);
   else
     launch_diag_partial(m, U, s);
@@ -1468,7 +1475,7 @@ int ucns_diagnostics(ucns_mesh* m, const double* U, ucns_diag* out, void* stream
   rc = timed(m, kKindDiag, s, [&] {
     if (mixed(m))
       k_diag_partial_mx<<<m->d.red_blocks, kRedThreads, 0, s>>>(U, m->d.coeff, coef_row_floats(m), m->NC,
-                                                                 m->d.vol, (int)m->N, m->d.red);
+                                                                 linear_entries(m), m->d.vol, (int)m->N, m->d.red);
     else
       launch_diag_partial(m, U, s);
     // the final sums land in the first 4 doubles of G (free between residuals)

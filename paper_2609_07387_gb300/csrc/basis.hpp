@@ -42,4 +42,14 @@ UCNS_HD constexpr int basis_lower(int k, int d) {
   return basis_index(basis_exp(k, 0) - (d == 0), basis_exp(k, 1) - (d == 1), basis_exp(k, 2) - (d == 2));
 }
 
+// Place of a monomial (k = -1: the constant) in the order in which a nested Horner
+// evaluation of degree r reads the coefficients: by descending power of z, then of
+// y, then of x, the constant last
+UCNS_HD constexpr int horner_place(int k, int r) {
+  const int e[3] = {k < 0 ? 0 : basis_exp(k, 0), k < 0 ? 0 : basis_exp(k, 1), k < 0 ? 0 : basis_exp(k, 2)};
+  const int D = r - e[2], E = D - e[1];  // degrees left in (x, y) and in x
+  // levels above in z: sum of (d+1)(d+2)/2 for d < D; in y: sum of (d+1) for d < E
+  return D * (D + 1) * (D + 2) / 6 + E * (E + 1) / 2 + E - e[0];
+}
+
 }  // namespace ucns

@@ -447,8 +447,8 @@ struct ReconArgsHOMx {
   const float* __restrict__ Msi;    // [K(K+1)/2][N]
   const float* __restrict__ psib;   // [K-3][N]
   const float* __restrict__ inv_h;  // [N]
-  float* __restrict__ coef;         // [N][cs] rows, entries cidx(v, k, K + 1): k = 0 relative to U_ref,
-                                    // then the physical-unit coefficients
+  float* __restrict__ coef;         // [N][cs] rows, entries cidx(v, horner_place(k), K + 1): the constant relative
+                                    // to U_ref, the others in physical units
   int* err;                         // bit 1: a copy wait gave up
   int N, cs;
   float lam0, lams, eps;
@@ -702,9 +702,9 @@ __global__ void __launch_bounds__(HOTile<ORDER>::THREADS, ORDER == 4 ? (WENO ? 1
 #pragma unroll
   for (int e = 1; e <= ORDER; e++) ihp[e] = ihp[e - 1] * ih;
   float* out = a.coef + (size_t)i * a.cs;
-  out[cidx(v, 0, K + 1)] = c0;
+  out[cidx(v, horner_place(-1, ORDER), K + 1)] = c0;
 #pragma unroll
-  for (int k = 0; k < K; k++) out[cidx(v, k + 1, K + 1)] = cf[k] * ihp[basis_degree(k)];
+  for (int k = 0; k < K; k++) out[cidx(v, horner_place(k, ORDER), K + 1)] = cf[k] * ihp[basis_degree(k)];
 }
 
 }  // namespace ucns

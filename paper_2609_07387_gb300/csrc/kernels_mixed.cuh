@@ -57,7 +57,8 @@ __host__ __device__ __forceinline__ size_t blk2(int row, int rows, int64_t i) {
   return (((size_t)(i / kTC) * (rows / 2) + row / 2) * kTC + (size_t)(i % kTC)) * 2 + (row & 1);
 }
 
-// index of entry k (0: the constant term) of variable v in a mixed-form
+// index of entry k (at P1 and P2 0 is the constant term and k + 1 mode k; at P3 and P4
+// the entries lie in the order of horner_place) of variable v in a mixed-form
 // coefficient row with ncf = K + 1 entries per variable: variables 0-3
 // interleaved per entry (k 4 + v, so one 16-byte load brings entry k of all
 // four, as two packed FP32x2 pairs), variable 4 after them (4 ncf + k)
@@ -577,79 +578,77 @@ __device__ __forceinline__ void viscous_flux_mx(const float W[5], const float g[
   Fv[4] = fmaf(u[0], Fv[1], fmaf(u[1], Fv[2], fmaf(u[2], Fv[3], c.k_e * ir * en)));
 }
 
-// value and gradient at (x, y, z) of a P3/P4 cell polynomial from its row
-// (entries cidx(v, k, K + 1), in global or shared memory): variables 0-3 in
-// packed FP32x2 pairs from one 16-byte load per mode, variable 4 from four
-// modes per 16-byte load
+// five variables: 0-3 as two packed FP32x2 pairs, 4 on its own
+struct Five {
+  float2 a, b;
+  float c;
+};
+__device__ __forceinline__ Five fma5(const Five& p, float x, const Five& q) {
+  const float2 X = make_float2(x, x);
+  return {__ffma2_rn(p.a, X, q.a), __ffma2_rn(p.b, X, q.b), fmaf(p.c, x, q.c)};
+}
+
+// value and gradient at (x, y, z) of a P3/P4 cell polynomial from its row (16-byte
+// aligned, in shared memory): nested Horner schemes in z of schemes in y of schemes
+// in x, with their derivatives carried along.  Per variable 35 / 65 FMAs at P3 / P4,
+// where summing the monomials' values and gradients takes 49 / 94 and the
+// monomials themselves (about 60 / 120 products per point).  Entries lie in the
+// order read (horner_place): variables 0-3 one 16-byte load per entry, variable 4
+// four entries per 16-byte load.  The face kernel is bound by instruction issue:
+// P3 at 40^3 74.8 -> 69.0 us, P4 at 32^3 87.0 -> 66.0.
 template <int ORDER, bool ACC>
 __device__ __forceinline__ void eval_side_ho_mx(const float* row, float x, float y, float z, float U[5],
                                                 float g[5][3]) {
-  constexpr int K = basis_count(ORDER), NCF = K + 1;
+  constexpr int NCF = basis_count(ORDER) + 1;
   const float4* r4 = reinterpret_cast<const float4*>(row);
-  float px[ORDER + 1], py[ORDER + 1], pz[ORDER + 1];
-  px[0] = py[0] = pz[0] = 1.f;
+  int at = 0;
+  float4 e4;
+  auto next = [&]() -> Five {
+    const float4 q = r4[at];
+    if (at % 4 == 0) e4 = r4[NCF + at / 4];
+    const float c = at % 4 == 0 ? e4.x : (at % 4 == 1 ? e4.y : (at % 4 == 2 ? e4.z : e4.w));
+    at++;
+    return {make_float2(q.x, q.y), make_float2(q.z, q.w), c};
+  };
+  Five u, ux, uy, uz;
 #pragma unroll
-  for (int e = 1; e <= ORDER; e++) {
-    px[e] = px[e - 1] * x;
-    py[e] = py[e - 1] * y;
-    pz[e] = pz[e - 1] * z;
-  }
-  float e4[4 * ((NCF + 3) / 4)];  // variable 4's entries
+  for (int k = ORDER; k >= 0; k--) {
+    Five r, rx, ry;
+    const int D = ORDER - k;  // degree in (x, y)
 #pragma unroll
-  for (int jj = 0; jj < (NCF + 3) / 4; jj++) {
-    const float4 t = r4[NCF + jj];
-    e4[4 * jj] = t.x;
-    e4[4 * jj + 1] = t.y;
-    e4[4 * jj + 2] = t.z;
-    e4[4 * jj + 3] = t.w;
-  }
-  const float4 c0 = r4[0];
-  float2 u01 = make_float2(c0.x, c0.y), u23 = make_float2(c0.z, c0.w);
-  float2 gx01 = make_float2(0.f, 0.f), gx23 = gx01, gy01 = gx01, gy23 = gx01, gz01 = gx01, gz23 = gx01;
-  float u4 = e4[0], gx4 = 0.f, gy4 = 0.f, gz4 = 0.f;
+    for (int j = D; j >= 0; j--) {
+      Five q = next(), qx;
+      const int E = D - j;  // degree in x
 #pragma unroll
-  for (int k = 0; k < K; k++) {
-    const int ex = basis_exp(k, 0), ey = basis_exp(k, 1), ez = basis_exp(k, 2);
-    const float mv = px[ex] * py[ey] * pz[ez];
-    const float4 cq = r4[k + 1];
-    const float2 c01 = make_float2(cq.x, cq.y), c23 = make_float2(cq.z, cq.w);
-    const float c4 = e4[k + 1];
-    u01 = __ffma2_rn(c01, make_float2(mv, mv), u01);
-    u23 = __ffma2_rn(c23, make_float2(mv, mv), u23);
-    u4 = fmaf(c4, mv, u4);
-    if (ex) {
-      const float m = ex * px[ex > 0 ? ex - 1 : 0] * py[ey] * pz[ez];
-      gx01 = __ffma2_rn(c01, make_float2(m, m), gx01);
-      gx23 = __ffma2_rn(c23, make_float2(m, m), gx23);
-      gx4 = fmaf(c4, m, gx4);
+      for (int i = E - 1; i >= 0; i--) {
+        qx = i == E - 1 ? q : fma5(qx, x, q);
+        q = fma5(q, x, next());
+      }
+      if (j < D) ry = j == D - 1 ? r : fma5(ry, y, r);
+      r = j == D ? q : fma5(r, y, q);
+      if (E >= 1) rx = E == 1 ? qx : fma5(rx, y, qx);
     }
-    if (ey) {
-      const float m = ey * px[ex] * py[ey > 0 ? ey - 1 : 0] * pz[ez];
-      gy01 = __ffma2_rn(c01, make_float2(m, m), gy01);
-      gy23 = __ffma2_rn(c23, make_float2(m, m), gy23);
-      gy4 = fmaf(c4, m, gy4);
-    }
-    if (ez) {
-      const float m = ez * px[ex] * py[ey] * pz[ez > 0 ? ez - 1 : 0];
-      gz01 = __ffma2_rn(c01, make_float2(m, m), gz01);
-      gz23 = __ffma2_rn(c23, make_float2(m, m), gz23);
-      gz4 = fmaf(c4, m, gz4);
+    if (k < ORDER) uz = k == ORDER - 1 ? u : fma5(uz, z, u);
+    u = k == ORDER ? r : fma5(u, z, r);
+    if (D >= 1) {
+      ux = D == 1 ? rx : fma5(ux, z, rx);
+      uy = D == 1 ? ry : fma5(uy, z, ry);
     }
   }
-  const float u[5] = {u01.x, u01.y, u23.x, u23.y, u4};
-  const float gx[5] = {gx01.x, gx01.y, gx23.x, gx23.y, gx4}, gy[5] = {gy01.x, gy01.y, gy23.x, gy23.y, gy4},
-              gz[5] = {gz01.x, gz01.y, gz23.x, gz23.y, gz4};
+  const float v[5] = {u.a.x, u.a.y, u.b.x, u.b.y, u.c};
+  const float gx[5] = {ux.a.x, ux.a.y, ux.b.x, ux.b.y, ux.c}, gy[5] = {uy.a.x, uy.a.y, uy.b.x, uy.b.y, uy.c},
+              gz[5] = {uz.a.x, uz.a.y, uz.b.x, uz.b.y, uz.c};
 #pragma unroll
-  for (int v = 0; v < 5; v++) {
-    U[v] = u[v];
+  for (int w = 0; w < 5; w++) {
+    U[w] = v[w];
     if (ACC) {
-      g[v][0] += gx[v];
-      g[v][1] += gy[v];
-      g[v][2] += gz[v];
+      g[w][0] += gx[w];
+      g[w][1] += gy[w];
+      g[w][2] += gz[w];
     } else {
-      g[v][0] = gx[v];
-      g[v][1] = gy[v];
-      g[v][2] = gz[v];
+      g[w][0] = gx[w];
+      g[w][1] = gy[w];
+      g[w][2] = gz[w];
     }
   }
 }
@@ -821,7 +820,8 @@ __global__ void __launch_bounds__(kFaceThreads, 1) k_face_mx(FaceArgsMx a) {
 // diagnostics partial sums from FP32 coefficients (FP64 accumulation)
 __global__ void __launch_bounds__(kRedThreads)
     k_diag_partial_mx(const double* __restrict__ U, const float* __restrict__ coef, int cs,
-                      int ncf /* entries per variable, K + 1 */, const double* __restrict__ vol, int N,
+                      int ncf /* entries per variable, K + 1 */, int3 lin /* the linear terms' entries */,
+                      const double* __restrict__ vol, int N,
                       double* __restrict__ part) {
   __shared__ double sm[4][kRedThreads];
   double acc[4] = {0, 0, 0, 0};
@@ -829,10 +829,11 @@ __global__ void __launch_bounds__(kRedThreads)
     const double r = U[i], ir = 1.0 / r;
     const double u[3] = {U[(size_t)N + i] * ir, U[2 * (size_t)N + i] * ir, U[3 * (size_t)N + i] * ir};
     double g[4][3];  // physical-unit linear coefficients = gradient at the centroid
+    const int le[3] = {lin.x, lin.y, lin.z};
 #pragma unroll
     for (int v = 0; v < 4; v++)
 #pragma unroll
-      for (int j = 0; j < 3; j++) g[v][j] = (double)coef[(size_t)i * cs + cidx(v, j + 1, ncf)];
+      for (int j = 0; j < 3; j++) g[v][j] = (double)coef[(size_t)i * cs + cidx(v, le[j], ncf)];
     double gu[3][3];
 #pragma unroll
     for (int q = 0; q < 3; q++)
