@@ -323,7 +323,7 @@ int launch_recon_tiles(const ReconArgsMx& a, cudaStream_t s) {
 template <int ORDER, bool WENO>
 int launch_recon_ho_tiles(const ReconArgsHOMx& a, cudaStream_t s) {
   using T = HOTile<ORDER>;
-  constexpr size_t sm = T::smem();
+  constexpr size_t sm = T::smem(WENO);
   UCNS_CUDA(cudaFuncSetAttribute(k_recon_ho_mx<ORDER, WENO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
   const unsigned g = (unsigned)((a.N + T::TC - 1) / T::TC);
   k_recon_ho_mx<ORDER, WENO><<<g, T::THREADS, sm, s>>>(a);

@@ -12,7 +12,7 @@
 //               the monomial-form polynomials, HLLC, penalised viscous flux
 //               (Eq. 7), and the face total summed by the group's first lane
 //               over its lanes in point order (deterministic).
-//   k_recon_ho_mx the same in the mixed form, tile by tile (64 cells): the
+//   k_recon_ho_mx the same in the mixed form, tile by tile (32 cells): the
 //               stencil ids and FP32 pseudo-inverses stream through shared
 //               memory in bulk-copied chunks, thread = (cell, variable).
 //   (the mixed face kernel of every order is k_face_mx, kernels_mixed.cuh)
@@ -443,7 +443,7 @@ __global__ void __launch_bounds__(kFaceHoThreads, 8) k_face_ho(FaceArgs a) {
 // face totals (k_rk<s, nfc, float> sums them as float pairs into FP64).
 struct ReconArgsHOMx {
   const float* __restrict__ Uhl;    // [N][5][2] float pairs (hi, lo) of the state
-  const float* __restrict__ tiles;  // per 64-cell tile its stencil chunks (HOTile)
+  const float* __restrict__ tiles;  // per 32-cell tile its stencil chunks (HOTile)
   const float* __restrict__ Msi;    // [K(K+1)/2][N]
   const float* __restrict__ psib;   // [K-3][N]
   const float* __restrict__ inv_h;  // [N]
@@ -455,31 +455,35 @@ struct ReconArgsHOMx {
   float eref_hi, eref_lo;  // E_ref = p_ref/(gamma-1) as a float pair
 };
 
-// The P3/P4 mixed reconstruction's data, tile by tile (64 cells): the central
+// The P3/P4 mixed reconstruction's data, tile by tile (32 cells): the central
 // stencil in NCC chunks of MCH members, then each of the six directional
-// stencils in NDC chunks of MDH members.  A chunk is [members][64] stencil ids
+// stencils in NDC chunks of MDH members.  A chunk is [members][32] stencil ids
 // (int32) followed by its pseudo-inverse entries as pairs of consecutive
-// members, [modes][members / 2][64][2]; every chunk is one bulk copy.  Cells
+// members, [modes][members / 2][32][2]; every chunk is one bulk copy.  Cells
 // past N in the last tile have ids 0 and zero entries.
 template <int ORDER>
 struct HOTile {
   using H = HO<ORDER>;
   static constexpr int K = H::K, MC = H::MC, KD = H::KD, MD = H::MD;
-  static constexpr int TC = 64;
+  static constexpr int TC = 32;
   static constexpr int MCH = ORDER == 4 ? 4 : 2, MDH = 6;
   static constexpr int NCC = MC / MCH, NDC = MD / MDH;
   static constexpr int CCS = MCH * TC + K * MCH * TC;  // floats per central chunk
   static constexpr int DCS = MDH * TC + KD * MDH * TC;  // floats per directional chunk
   static constexpr int CENTRAL = NCC * CCS;
   static constexpr int STAGE = CCS > DCS ? CCS : DCS;
-  // with CWENOZ the smoothness matrices follow the central chunks: [K(K+1)/2][64]
+  // with CWENOZ the smoothness matrices follow the central chunks: [K(K+1)/2][32]
   // entries in chunks of MSR rows, then the directional chunks
   static constexpr int NQS = K * (K + 1) / 2, MSR = STAGE / TC, NMC = (NQS + MSR - 1) / MSR;
   static constexpr int SMAT = NQS * TC;
   UCNS_HD static constexpr int tile_floats(bool weno) { return CENTRAL + (weno ? SMAT + 6 * NDC * DCS : 0); }
   static constexpr int S = ORDER == 4 ? 3 : 4;  // stages of the copy ring (6 at P4 measured slower)
   static constexpr int THREADS = 5 * TC + 32;   // (cell, variable) threads and one copying warp
-  static constexpr size_t smem() { return (size_t)S * STAGE * 4 + (size_t)2 * S * 8; }
+  // the ring, its barriers, then (CWENOZ) the directional candidates, one column per thread
+  static constexpr size_t smem(bool weno) {
+    return (size_t)S * STAGE * 4 + (size_t)2 * S * 8 + (weno ? (size_t)6 * KD * 5 * TC * 4 : 0);
+  }
+  static constexpr int blocks(bool weno) { return ORDER == 4 ? (weno ? 2 : 4) : 4; }
   static_assert(MC % MCH == 0 && MD % MDH == 0 && MCH % 2 == 0 && MDH % 2 == 0, "whole member pairs");
   static_assert(CCS % 4 == 0 && DCS % 4 == 0, "16-byte chunks");
 };
@@ -509,7 +513,7 @@ __device__ __forceinline__ float pair_diff_ho(const float* __restrict__ hl, int 
 template <int KK, int MM>
 __device__ __forceinline__ void chunk_contract(const float* chunk, int c, const float* __restrict__ hl, int v,
                                                float hi_i, float lo_i, float (&acc)[KK]) {
-  constexpr int TC = 64;
+  constexpr int TC = 32;
   const float2* P = reinterpret_cast<const float2*>(chunk + MM * TC);
 #pragma unroll
   for (int mp = 0; mp < MM / 2; mp++) {
@@ -524,24 +528,25 @@ __device__ __forceinline__ void chunk_contract(const float* chunk, int c, const 
   }
 }
 
-// One block per 64-cell tile: thread (cell c, variable v) = 5 c + v, plus a
+// One block per 32-cell tile: thread (cell c, variable v) = 5 c + v, plus a
 // copying warp that streams the tile's chunks (central; with CWENOZ the
-// smoothness matrices, then the directional chunks twice, once for the
-// indicators and once for the combination) through a ring of S shared-memory
-// stages, every wait bounded.
-// Per variable the arithmetic is that of the FP64 form in FP32, members and
-// modes in the same order.  Blocks per SM: P3 three, P4 two (linear) or one
-// (CWENOZ: 168 registers a thread without spills; two blocks at 80 registers
-// spill and measured no faster).
+// smoothness matrices, then the directional chunks) through a ring of S
+// shared-memory stages, every wait bounded; the directional candidates wait in
+// shared memory for the weights.  Per variable the arithmetic is that of the
+// FP64 form in FP32, members and modes in the same order.  Bound by the latency of
+// the state gathers.  CWENOZ at P3 40^3 / P4 32^3, us: 64-cell tiles, the directional
+// chunks streamed and contracted twice 89 / 182, 32-cell tiles 88 / 166, the candidates
+// kept 79 / 158 (P3 at 4, 5, 6 blocks per SM 79, 82, 87; P4 at 1 and 2 173, 158).
 template <int ORDER, bool WENO>
-__global__ void __launch_bounds__(HOTile<ORDER>::THREADS, ORDER == 4 ? (WENO ? 1 : 2) : 3) k_recon_ho_mx(ReconArgsHOMx a) {
+__global__ void __launch_bounds__(HOTile<ORDER>::THREADS, HOTile<ORDER>::blocks(WENO)) k_recon_ho_mx(ReconArgsHOMx a) {
   using T = HOTile<ORDER>;
   constexpr int K = T::K, KD = T::KD, ND = 6, TC = T::TC, S = T::S;
-  constexpr int NQ = T::NCC + (WENO ? T::NMC + 2 * ND * T::NDC : 0);  // chunks streamed per tile
+  constexpr int NQ = T::NCC + (WENO ? T::NMC + ND * T::NDC : 0);  // chunks streamed per tile
   extern __shared__ __align__(128) unsigned char smem[];
   float* st = reinterpret_cast<float*>(smem);
   uint64_t* full = reinterpret_cast<uint64_t*>(st + S * T::STAGE);
   uint64_t* empty = full + S;
+  float* sB = reinterpret_cast<float*>(empty + S) + threadIdx.x;  // this thread's column of candidates
   const int t = threadIdx.x, lane = t & 31, tile = blockIdx.x;
   if (t < S) {
     bar_init(&full[t]);
@@ -558,7 +563,7 @@ __global__ void __launch_bounds__(HOTile<ORDER>::THREADS, ORDER == 4 ? (WENO ? 1
         ok = false;
         break;
       }
-      // chunk q: central chunks first, then the directional ones in two rounds
+      // chunk q: central chunks first, then the smoothness matrices, then the directional ones
       const float* src;
       uint32_t bytes;
       if (q < T::NCC) {
@@ -569,7 +574,7 @@ __global__ void __launch_bounds__(HOTile<ORDER>::THREADS, ORDER == 4 ? (WENO ? 1
         src = base + T::CENTRAL + (size_t)r0 * TC;
         bytes = (uint32_t)(min(T::MSR, T::NQS - r0) * TC) * 4u;
       } else {
-        const int qd = (q - T::NCC - T::NMC) % (ND * T::NDC);
+        const int qd = q - T::NCC - T::NMC;
         src = base + T::CENTRAL + T::SMAT + (size_t)qd * T::DCS;
         bytes = T::DCS * 4u;
       }
@@ -653,6 +658,8 @@ __global__ void __launch_bounds__(HOTile<ORDER>::THREADS, ORDER == 4 ? (WENO ? 1
         chunk_contract<KD, T::MDH>(chunk, c, hl, v, hi_i, lo_i, b);
         give();
       }
+#pragma unroll
+      for (int k = 0; k < KD; k++) sB[(s * KD + k) * 5 * TC] = b[k];
       SI[s] = si_form_f<K, KD>(a.Msi, N, i, b);
       tau += fabsf(SI0 - SI[s]);
     }
@@ -669,21 +676,11 @@ __global__ void __launch_bounds__(HOTile<ORDER>::THREADS, ORDER == 4 ? (WENO ? 1
     const float r0 = fdiv(w0 * iws, a.lam0);
 #pragma unroll
     for (int k = 0; k < K; k++) cf[k] = r0 * ao[k];
-#pragma unroll 1
-    for (int s = 0; s < ND && ok; s++) {
-      float b[KD];
 #pragma unroll
-      for (int k = 0; k < KD; k++) b[k] = 0.f;
-#pragma unroll 1
-      for (int h = 0; h < T::NDC; h++) {
-        const float* chunk = take();
-        if (!ok) break;
-        chunk_contract<KD, T::MDH>(chunk, c, hl, v, hi_i, lo_i, b);
-        give();
-      }
+    for (int s = 0; s < ND; s++) {
       const float e = ws[s] * iws - r0 * a.lams;
 #pragma unroll
-      for (int k = 0; k < KD; k++) cf[k] = fmaf(e, b[k], cf[k]);
+      for (int k = 0; k < KD; k++) cf[k] = fmaf(e, sB[(s * KD + k) * 5 * TC], cf[k]);
     }
   }
   if (!ok) {

@@ -33,8 +33,10 @@ struct FluxConstF {
 // tiles of kTC consecutive (Morton-ordered) cells, and for every tile all rows
 // of an array [rows][kTC] contiguous, so that one bulk copy brings a tile's
 // pseudo-inverse rows (or stencil lists) into shared memory.  Cells past N in
-// the last tile are zero rows.
-constexpr int kTC = 64;
+// the last tile are zero rows.  Four (CWENOZ) or six tiles per SM overlap copies and
+// arithmetic better than two or three of 64 cells: k_recon_mx at 96^3 334 -> 321 us
+// (CWENOZ), 190 -> 183 (gated), tetrahedra (453,600) 161 -> 153; of 16 cells 341, 191, 151.
+constexpr int kTC = 32;
 
 // FP32 division and square root of the mixed form: the hardware approximate
 // reciprocal and reciprocal square root (at most 2 ulp: CUDA's __fdividef and
@@ -315,7 +317,7 @@ __device__ __forceinline__ void gated_cwenoz(const ReconArgsMx& a, const float (
 // bulk copy.  GATED (WENO = false, P2): a gated CWENOZ reconstruction, linear
 // weights for every cell first, then gated_cwenoz for the flagged ones.
 template <int ORDER, bool WENO, int ND, bool GATED>
-__global__ void __launch_bounds__(kTC * 5, WENO ? 2 : 3) k_recon_mx(ReconArgsMx a) {
+__global__ void __launch_bounds__(kTC * 5, WENO ? 4 : 6) k_recon_mx(ReconArgsMx a) {
   using T = ReconTile<ORDER, WENO, ND>;
   constexpr int K = T::K, MC = T::MC, MD = T::MD, CS = T::CS;
   extern __shared__ __align__(128) unsigned char smem[];

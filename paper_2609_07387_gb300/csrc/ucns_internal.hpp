@@ -38,13 +38,13 @@ struct DeviceMesh {
   int32_t* fx_ids = nullptr;     // FP64 form at P3/P4: [tiles][IDS][24] stencils
   int16_t* fx_exps = nullptr;    // [tiles][EXPS][24] row exponents
   double* Msi = nullptr;      // P3/P4: [K(K+1)/2][N] smoothness-indicator matrix (upper triangle, row-major)
-  float* hot = nullptr;       // P3/P4 mixed form: stencil ids and FP32 pseudo-inverses in 64-cell tiles; FP32 Msi, psib
+  float* hot = nullptr;       // P3/P4 mixed form: stencil ids and FP32 pseudo-inverses in 32-cell tiles; FP32 Msi, psib
   float* Msif = nullptr;
   float* psibf = nullptr;
   double* psib = nullptr;     // P3/P4: [K-3][N] cell means of the non-linear basis monomials (xi units)
   // mixed precision: FP32 pseudo-inverses and the stencils in the pair-blocked
-  // layout [ceil(N/64)][rows/2][64][2] (tiles of 64 consecutive cells, row
-  // pairs of a cell adjacent), the cell rows blocked [ceil(N/64)][rows][64]
+  // layout [ceil(N/32)][rows/2][32][2] (tiles of 32 consecutive cells, row
+  // pairs of a cell adjacent), the cell rows blocked [ceil(N/32)][rows][32]
   float* Pcb = nullptr;       // rows k Mc + m
   float* Pdb = nullptr;       // rows (s 3 + k) Md + r
   int32_t* scb = nullptr;     // rows m
