@@ -107,7 +107,10 @@ struct RKArgs {
 // for the fewest FP64 operations: two divisions less than the difference form of
 // the star flux and Roe's enthalpy, 1/rho once in the viscous flux, the energy
 // gradient by its normal part (k_face<2> at 72 x 80 x 88 5418 -> 4756 us; the mixed
-// form's fluxes, written alike, k_face_mx<2> at 96^3 210 -> 196 us).
+// form's fluxes, written alike, k_face_mx<2> at 96^3 210 -> 196 us).  With integer
+// evaluation: the penalty jump as one FMA a component, sign tests on the bits and
+// the face sum shared out among the lanes, 2974 -> 2839 us (P4 at 24^3, whose points were
+// summed by every lane, 534 -> 454).
 __device__ __forceinline__ void phys_flux(const double U[5], const double u[3], double p,
                                           double un, const double n[3], double F[5]) {
   F[0] = U[0] * un;
@@ -131,6 +134,13 @@ __device__ __forceinline__ void star_flux(const double U[5], double ir, const do
   // rho* (E/rho + (Ss - u_n)(Ss + p/m)), rho*/m = r
   const double Es = fma(rho, fma(ds, Ss, U[4] * ir), (ds * p) * r);
   F[4] = Ss * (Es + ps);
+}
+
+// x >= 0 (true for -0, false for NaN) from the bit pattern
+__device__ __forceinline__ bool not_below_zero(double x) {
+  const int hi = __double2hiint(x), lo = __double2loint(x);
+  const bool nan = (hi & 0x7fffffff) > 0x7ff00000 || ((hi & 0x7fffffff) == 0x7ff00000 && lo != 0);
+  return (hi >= 0 || ((hi & 0x7fffffff) | lo) == 0) && !nan;
 }
 
 // HLLC (Toro, Spruce & Speares) with Einfeldt/Roe wave-speed bounds; flux
@@ -162,40 +172,44 @@ __device__ __forceinline__ void hllc_flux(const double UL[5], const double UR[5]
   const double SR = fmax(unR + aR, utn + at);
   const double mL = rL * (SL - unL), mR = rR * (SR - unR);
   const double Ss = (pR - pL + unL * mL - unR * mR) / (mL - mR);
-  if (0.0 <= SL) {
+  if (not_below_zero(SL)) {
     phys_flux(UL, uL, pL, unL, n, F);
-  } else if (0.0 <= Ss) {
+  } else if (not_below_zero(Ss)) {
     star_flux(UL, irL, uL, pL, unL, mL, SL, Ss, n, F);
-  } else if (0.0 <= SR) {
+  } else if (not_below_zero(SR)) {
     star_flux(UR, irR, uR, pR, unR, mR, SR, Ss, n, F);
   } else {
     phys_flux(UR, uR, pR, unR, n, F);
   }
 }
 
-// Viscous flux F_v . n from a face state (up to a common factor with g) and the
-// conserved gradients: g of density and momenta, g4n = grad(rho E) . n.  Written
-// with rho grad u = grad m - u grad rho, so that the one 1/rho enters at the end:
-//   t_a = (mu/rho)(G_aj n_j + G_ja n_j - 2/3 tr(G) n_a),  G = rho grad u
-//   rho grad e . n = grad(rho E) . n - E grad rho . n - u_a G_aj n_j
-__device__ __forceinline__ void viscous_flux(const double U[5], const double g[4][3], double g4n,
+// Viscous flux F_v . n of the face state U and the penalised gradient g + J n (both up
+// to a common factor): g of density, momenta and energy, J the penalised jumps.
+// Written with rho grad u = grad m - u grad rho = S + K n, S = g_m - u g_rho and K = J_m
+// - u J_rho, so that the one 1/rho enters at the end and the jump costs one FMA each:
+//   t_a = (mu/rho)(S_aj n_j + K_a + S_ja n_j + (K.n - 2/3 (tr S + K.n)) n_a)
+//   rho grad e . n = (g_E . n + J_E) - E/rho (g_rho . n + J_rho) - u_a (S_aj n_j + K_a)
+__device__ __forceinline__ void viscous_flux(const double U[5], const double g[5][3], const double J[5],
                                              const double n[3], const FluxConst& c, double Fv[5]) {
   const double ir = 1.0 / U[0];
   const double u[3] = {U[1] * ir, U[2] * ir, U[3] * ir};
-  double G[3][3], dn[3];
+  double S[3][3], K[3], dn[3];
 #pragma unroll
   for (int a = 0; a < 3; a++) {
+    K[a] = fma(-u[a], J[0], J[1 + a]);
 #pragma unroll
-    for (int j = 0; j < 3; j++) G[a][j] = fma(-u[a], g[0][j], g[1 + a][j]);
-    dn[a] = fma(G[a][0], n[0], fma(G[a][1], n[1], G[a][2] * n[2]));
+    for (int j = 0; j < 3; j++) S[a][j] = fma(-u[a], g[0][j], g[1 + a][j]);
+    dn[a] = fma(S[a][0], n[0], fma(S[a][1], n[1], fma(S[a][2], n[2], K[a])));
   }
-  const double tdiv = (2.0 / 3.0) * (G[0][0] + G[1][1] + G[2][2]);
+  const double Kn = fma(K[0], n[0], fma(K[1], n[1], K[2] * n[2]));
+  const double w = fma(-2.0 / 3.0, S[0][0] + S[1][1] + S[2][2], (1.0 / 3.0) * Kn);  // K.n - 2/3 (tr S + K.n)
   const double mr = c.mu * ir;
   Fv[0] = 0.0;
 #pragma unroll
   for (int a = 0; a < 3; a++)
-    Fv[1 + a] = mr * fma(G[0][a], n[0], fma(G[1][a], n[1], fma(G[2][a], n[2], fma(-tdiv, n[a], dn[a]))));
-  const double g0n = fma(g[0][0], n[0], fma(g[0][1], n[1], g[0][2] * n[2]));
+    Fv[1 + a] = mr * fma(S[0][a], n[0], fma(S[1][a], n[1], fma(S[2][a], n[2], fma(w, n[a], dn[a]))));
+  const double g0n = fma(g[0][0], n[0], fma(g[0][1], n[1], fma(g[0][2], n[2], J[0])));
+  const double g4n = fma(g[4][0], n[0], fma(g[4][1], n[1], fma(g[4][2], n[2], J[4])));
   const double en = fma(-u[0], dn[0], fma(-u[1], dn[1], fma(-u[2], dn[2], fma(-(U[4] * ir), g0n, g4n))));
   Fv[4] = fma(u[0], Fv[1], fma(u[1], Fv[2], fma(u[2], Fv[3], c.k_e * ir * en)));
 }
@@ -204,24 +218,20 @@ __device__ __forceinline__ void viscous_flux(const double U[5], const double g[4
 // grad U_L + grad U_R: HLLC, less (VISC) the viscous flux of the penalised face
 // gradient.  2 U_f = U_L + U_R and 2 grad U_f = gs + 2 (alpha/L)(U_R - U_L) n:
 // the viscous flux depends on them only through ratios, so the common factor 2
-// cancels; the energy gradient enters through its normal part alone.
+// cancels.
 template <bool VISC>
 __device__ __forceinline__ void point_flux(const double UL[5], const double UR[5], const double gs[5][3],
                                            const double n[3], double pen2, const FluxConst& c, double F[5]) {
   hllc_flux(UL, UR, n, c, F);
   if (VISC) {
-    double Uf2[5], gf2[4][3];
+    double Uf2[5], J[5];
 #pragma unroll
-    for (int v = 0; v < 4; v++) {
-      const double jump2 = pen2 * (UR[v] - UL[v]);
+    for (int v = 0; v < 5; v++) {
+      J[v] = pen2 * (UR[v] - UL[v]);
       Uf2[v] = UL[v] + UR[v];
-#pragma unroll
-      for (int j = 0; j < 3; j++) gf2[v][j] = fma(jump2, n[j], gs[v][j]);
     }
-    Uf2[4] = UL[4] + UR[4];
-    const double g4n = fma(gs[4][0], n[0], fma(gs[4][1], n[1], fma(gs[4][2], n[2], pen2 * (UR[4] - UL[4]))));
     double Fv[5];
-    viscous_flux(Uf2, gf2, g4n, n, c, Fv);
+    viscous_flux(Uf2, gs, J, n, c, Fv);
 #pragma unroll
     for (int v = 1; v < 5; v++) F[v] -= Fv[v];
   }
@@ -626,13 +636,27 @@ __global__ void __launch_bounds__(64, 8) k_face(FaceArgs a) {
   point_flux<VISC && !BND>(UL, UR, gs, n, VISC && !BND ? 2.0 * a.fpen[fc] : 0.0, a.c, flux);
 #pragma unroll
   for (int v = 0; v < 5; v++) flux[v] *= area;
+  if constexpr (NQ == 1) {
+    if (live) {
 #pragma unroll
-  for (int off = 1; off < NQ; off <<= 1)
-#pragma unroll
-    for (int v = 0; v < 5; v++) flux[v] += __shfl_xor_sync(0xffffffffu, flux[v], off);
-  if (live && q == 0) {
-#pragma unroll
-    for (int v = 0; v < 5; v++) a.G[(size_t)v * F + f] = flux[v];
+      for (int v = 0; v < 5; v++) a.G[(size_t)v * F + f] = flux[v];
+    }
+  } else {
+    // (q0 + q1) + (q2 + q3), the variables shared out among the four lanes: lanes 0 and
+    // 2 keep variables 0, 1, 4 of the first sums, lanes 1 and 3 variables 2, 3; then 0: 0
+    // and 4, 2: 1, 1: 2, 3: 3 (five FP64 additions a warp instead of ten)
+    const bool odd = q & 1, high = q & 2;
+    auto swap = [](double x, int off) { return __shfl_xor_sync(0xffffffffu, x, off); };
+    double s0 = swap(odd ? flux[0] : flux[2], 1), s1 = swap(odd ? flux[1] : flux[3], 1), s4 = swap(flux[4], 1);
+    s0 += odd ? flux[2] : flux[0];
+    s1 += odd ? flux[3] : flux[1];
+    s4 += flux[4];
+    const double t = swap(high ? s0 : s1, 2), t4 = swap(s4, 2);
+    const double x = (high ? s1 : s0) + t, x4 = s4 + t4;
+    if (live) {
+      a.G[(size_t)((odd ? 2 : 0) + (high ? 1 : 0)) * F + f] = x;
+      if (q == 0) a.G[4 * F + f] = x4;
+    }
   }
 }
 

@@ -418,21 +418,19 @@ __global__ void __launch_bounds__(kFaceHoThreads, 8) k_face_ho(FaceArgs a) {
   point_flux<VISC>(UL, UR, gs, n, VISC ? 2.0 * a.fpen[fc] : 0.0, a.c, flux);
 #pragma unroll
   for (int v = 0; v < 5; v++) flux[v] *= area;
-  // the group's first lane sums its NQ points in point order (every lane takes
-  // part in the shuffles; lanes outside a group read group 0 and store nothing)
-  const int base = (in_group ? grp : 0) * NQ;
-  double tot[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+  // each (face, variable) of the warp on a lane of its own, summed in point order
 #pragma unroll
-  for (int t = 0; t < NQ; t++)
+  for (int v = 0; v < 5; v++) sv[v][t] = flux[v];
+  __syncwarp();
+  const int g = lane / 5, v = lane - 5 * (lane / 5), fs = gw * FPW + g;
+  if (g < FPW && fs < a.F) {
+    const double* x = &sv[v][(t & ~31) + g * NQ];
+    double tot = x[0];
 #pragma unroll
-    for (int v = 0; v < 5; v++) tot[v] += __shfl_sync(0xffffffffu, flux[v], base + t);
-  if (live && q == 0) {
-#pragma unroll
-    for (int v = 0; v < 5; v++) a.G[(size_t)v * F + f] = tot[v];
+    for (int k = 1; k < NQ; k++) tot += x[k];
+    a.G[(size_t)v * F + fs] = tot;
   }
 }
-
-
 
 // ------------------------------------------------------- mixed P3 / P4
 // The mixed form at P3 / P4 (the arithmetic split of the mixed form at P2):
