@@ -748,6 +748,19 @@ __device__ __forceinline__ void split_pair(double u, float& hi, float& lo) {
   lo = t >= 0x7f800000u ? 0.f : (float)r * __uint_as_float(((eu - 948u) << 23) | sgn);
 }
 
+// FP64 rounded to FP32 by integer operations (as split_pair's hi); results outside the
+// normal FP32 range by the hardware conversion
+__device__ __forceinline__ float d2f(double u) {
+  const unsigned long long ub = (unsigned long long)__double_as_longlong(u);
+  const unsigned eu = (unsigned)(ub >> 52) & 0x7ffu;
+  if (eu - 897u > 1150u - 897u) return __double2float_rn(u);
+  const unsigned long long x = (ub & 0x7fffffffffffffffull) - (896ull << 52);
+  const unsigned rem = (unsigned)x & 0x1fffffffu;
+  const unsigned t = (unsigned)(x >> 29);
+  const bool up = rem > 0x10000000u || (rem == 0x10000000u && (t & 1u));
+  return __uint_as_float((t + (up ? 1u : 0u)) | ((unsigned)(ub >> 32) & 0x80000000u));
+}
+
 // rho > 0 and p > 0 (p > 0  <=>  2 rho E - |m|^2 > 0 for rho > 0), all finite
 __device__ __forceinline__ bool physical(const double U[5]) {
   const double q = 2.0 * U[0] * U[4] - (U[1] * U[1] + U[2] * U[2] + U[3] * U[3]);
