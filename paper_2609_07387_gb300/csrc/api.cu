@@ -125,6 +125,19 @@ int upload_fx_tiles(const ucns_mesh* m, const HostArrays& h, unsigned char** dst
   return upload(dst, b);
 }
 
+// the smoothness-indicator matrices' leading Kd x Kd block, upper triangle by rows
+std::vector<double> leading_block(const ucns_mesh* m, const HostArrays& h) {
+  const int K = m->K, Kd = m->Kd;
+  const int64_t N = m->N;
+  std::vector<double> b;
+  b.reserve((size_t)Kd * (Kd + 1) / 2 * N);
+  for (int k = 0; k < Kd; k++) {
+    const auto row = h.Msi.begin() + (size_t)(k * K - k * (k - 1) / 2) * N;
+    b.insert(b.end(), row, row + (size_t)(Kd - k) * N);
+  }
+  return b;
+}
+
 // the P3/P4 reconstruction's tiles (HOFxTile) of the FP64 form, their stencils and row exponents
 template <int ORDER>
 int upload_ho_fx_tiles(const ucns_mesh* m, const HostArrays& h, DeviceMesh& d) {
@@ -1276,7 +1289,8 @@ static int device_upload(ucns_mesh* m, const ucns_params* p, HostArrays& h) {
              (m->K == 3 && (rc = upload(&d.fq, h.fq))) ||
              (m->K > 3 && ((rc = upload_fixed_faces(m, &d.fq, &d.hexp, h.fq)) ||
                             (rc = alloc(&d.cexp, (size_t)5 * m->N)))) ||
-             (rc = upload(&d.fpen, h.fpen)) || (rc = upload(&d.Msi, h.Msi)) || (rc = upload(&d.psib, h.psib)) ||
+             (rc = upload(&d.fpen, h.fpen)) || (m->K > 9 && (rc = upload(&d.Msi, leading_block(m, h)))) ||
+             (rc = upload(&d.psib, h.psib)) ||
              (rc = alloc(&d.coef, (size_t)m->NC * m->N * 5))) {
     device_free(m);
     return rc;

@@ -22,9 +22,10 @@
 // hi'| <= 2^30 2^29 + M 2^29 2^(B - 30) < 2^63, so no accumulator overflows for
 // the M <= 68 members of a stencil.
 //
-// Error of a sum against the exact one, in units of max|d| sum|P|: operand
-// rounding 2^-(B + 1), row rounding M 2^-61, dropped terms M 2^-60 (all of random
-// sign).  An FP64 sum of M products rounds each partial sum to 2^-53 of itself.
+// Error of a sum against the exact one, in units of max|d| sum|P|: operand rounding
+// at most 2^-B, row rounding M 2^-59, dropped terms M 2^-57 (all of random sign, so
+// that about sqrt(M) 2^-60 is seen).  An FP64 sum of M products rounds each partial sum
+// to 2^-53 of itself.
 // Measured against 128 bits on random rows and operands of one magnitude, error
 // over sum|P d|, rms (largest): M = 18 fixed 1.9e-17 (9e-17), FP64 5.6e-17 (4.4e-16);
 // M = 68 fixed 1.6e-17 (1.1e-16), FP64 5.7e-17 (4.8e-16).

@@ -1,11 +1,13 @@
 // CUDA kernels of the residual / SSP-RK3 hot path (sm_103a).
 //
-//   k_recon   cell x variable parallel: stencil differences, least-squares
-//             contractions (Eq. 4), smoothness indicators and CWENOZ weights
-//             (Eqs. 5-6); writes monomial coefficients of the final polynomial.
+//   k_recon   tile by tile, cell x variable parallel: stencil differences and
+//             least-squares contractions (Eq. 4) in fixed point (fixed.cuh),
+//             smoothness indicators and CWENOZ weights (Eqs. 5-6) in FP64;
+//             writes monomial coefficients of the final polynomial.
 //   k_face    face x Gauss-point parallel: polynomial values and gradients at
-//             the point from both sides, HLLC flux, penalised viscous flux
-//             (Eq. 7), Gauss sum over the face by warp shuffles (fixed order).
+//             the point from both sides (fixed point from P2 on), HLLC flux,
+//             penalised viscous flux (Eq. 7), Gauss sum over the face by warp
+//             shuffles (fixed order).
 //   k_rk      cell parallel: owner-side residual of Eq. 2 (faces in fixed
 //             order, no atomics) fused with one SSP-RK3 stage.
 //   k_dt_*, k_diag_*: deterministic block-tree reductions.

@@ -71,7 +71,7 @@ struct ReconArgsHO {
   const unsigned char* __restrict__ tiles;  // records (HOFxTile)
   const int32_t* __restrict__ ids;          // [tiles][IDS][24]
   const int16_t* __restrict__ exps;         // [tiles][EXPS][24]
-  const double* __restrict__ Msi;   // [K(K+1)/2][N]: smoothness-indicator matrix, upper triangle by rows
+  const double* __restrict__ Msi;   // [KD(KD+1)/2][N]: the smoothness-indicator matrix's leading block, upper triangle by rows
   const double* __restrict__ psib;  // [K-3][N]: cell means of the basis monomials of degree >= 2
   const double* __restrict__ inv_h; // [N]
   const short4* __restrict__ hexp;  // [N] exponents of the cell's axis scales
@@ -82,16 +82,16 @@ struct ReconArgsHO {
   double lam0, lams, eps;
 };
 
-// a^T M a over the first KK modes (M: K x K symmetric, upper triangle stored
-// by rows: entry (k, l >= k) at q = k K - k (k - 1) / 2 + l - k)
-template <int K, int KK>
-__device__ __forceinline__ double si_form(const double* __restrict__ M, size_t N, int i, const double (&a)[KK]) {
+// a^T M a (M: K x K symmetric, upper triangle stored by rows: entry (k, l >= k) at
+// q = k K - k (k - 1) / 2 + l - k)
+template <int K>
+__device__ __forceinline__ double si_form(const double* __restrict__ M, size_t N, int i, const double (&a)[K]) {
   double s = 0.0;
 #pragma unroll
-  for (int k = 0; k < KK; k++) {
+  for (int k = 0; k < K; k++) {
     double t = 0.0;
 #pragma unroll
-    for (int l = k + 1; l < KK; l++) t = fma(__ldg(&M[(size_t)(k * K - k * (k - 1) / 2 + l - k) * N + i]), a[l], t);
+    for (int l = k + 1; l < K; l++) t = fma(__ldg(&M[(size_t)(k * K - k * (k - 1) / 2 + l - k) * N + i]), a[l], t);
     const double mkk = __ldg(&M[(size_t)(k * K - k * (k - 1) / 2) * N + i]);
     s = fma(a[k], fma(2.0, t, mkk * a[k]), s);
   }
@@ -310,7 +310,7 @@ __global__ void __launch_bounds__(HOFxTile<ORDER>::THREADS, 2) k_recon_ho(ReconA
       if (!ok) break;
 #pragma unroll
       for (int k = 0; k < KD; k++) sB[(s * KD + k) * L] = b[k];
-      SI[s] = si_form<K, KD>(a.Msi, N, i, b);
+      SI[s] = si_form<KD>(a.Msi, N, i, b);
       tau += fabs(SI0 - SI[s]);
     }
     tau *= (1.0 / ND);
@@ -486,7 +486,7 @@ struct HOTile {
   static_assert(CCS % 4 == 0 && DCS % 4 == 0, "16-byte chunks");
 };
 
-// a^T M a over the first KK modes of one variable (M as in si_form), FP32
+// a^T M a over the first KK modes of one variable (M: K x K, stored as in si_form), FP32
 template <int K, int KK>
 __device__ __forceinline__ float si_form_f(const float* __restrict__ M, size_t N, int i, const float (&a)[KK]) {
   float s = 0.f;

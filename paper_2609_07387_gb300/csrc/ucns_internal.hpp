@@ -37,7 +37,7 @@ struct DeviceMesh {
   unsigned char* fxt = nullptr;  // FP64 form from P2 on: least-squares rows in fixed point, tile by tile (P2: and stencils)
   int32_t* fx_ids = nullptr;     // FP64 form at P3/P4: [tiles][IDS][24] stencils
   int16_t* fx_exps = nullptr;    // [tiles][EXPS][24] row exponents
-  double* Msi = nullptr;      // P3/P4: [K(K+1)/2][N] smoothness-indicator matrix (upper triangle, row-major)
+  double* Msi = nullptr;      // FP64 form at P3/P4: [Kd(Kd+1)/2][N] leading block of the smoothness-indicator matrix
   float* hot = nullptr;       // P3/P4 mixed form: stencil ids and FP32 pseudo-inverses in 32-cell tiles; FP32 Msi, psib
   float* Msif = nullptr;
   float* psibf = nullptr;
