@@ -1,0 +1,106 @@
+"""The fixed-point sums of csrc/fixed.cuh on the host, against exact rational
+arithmetic: differences, contractions and conversions of FP64 values of one
+magnitude, of mixed ones, subnormal and near the largest, and non-finite ones.
+The bounds are those of the header: a sum is off by at most (2^-57 + M 2^-56.5)
+sum|P| max|u_m - u_0| and the final rounding."""
+import os
+import shutil
+import subprocess
+from fractions import Fraction
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2609_07387_gb300", "csrc")
+
+PROGRAM = r"""
+#include "fixed.cuh"
+#include <cstdio>
+#include <random>
+using namespace ucns;
+std::mt19937_64 g(5);
+double u() { return 2.0 * (double)(g() >> 11) / 9007199254740992.0 - 1.0; }
+template <int M> void sums(double scale, double spread) {
+  for (int t = 0; t < 40; t++) {
+    double P[M], U[M], l1 = 0.0, u0 = scale * (1.0 + spread * u());
+    for (int m = 0; m < M; m++) {
+      P[m] = u() * std::exp(2.0 * u());
+      U[m] = scale * (1.0 + spread * u());
+      l1 += std::fabs(P[m]);
+    }
+    printf("sum %d %a", M, u0);
+    for (int m = 0; m < M; m++) printf(" %a %a", P[m], U[m]);
+    const int E = fx_row_exponent(l1);
+    int2 q[M];
+    int e;
+    fx_differences<M>(U, u0, q, e);
+    FxAcc acc;
+    for (int m = 0; m < M; m++) fx_mac(acc, fx_limbs(fx_round(std::ldexp(P[m], 60 - E))), q[m]);
+    printf(" %a\n", fx_double(fx_sum(acc), E + e - 2 - fx_bits_of(M)));
+  }
+}
+int main() {
+  for (double spread : {1e-9, 0.1, 10.0})
+    for (double scale : {1.0, 1e-200, 1e200, 0x1p-1000}) { sums<6>(scale, spread); sums<18>(scale, spread); sums<68>(scale, spread); }
+  for (int t = 0; t < 4000; t++) {
+    const long long s = (long long)g() >> (g() % 63);
+    const int e = (int)(g() % 2100) - 1080;
+    printf("double %lld %d %a\n", s, e, fx_double(s, e));
+    const double a = u() * std::ldexp(1.0, (int)(g() % 200) - 100), b = u() * std::ldexp(1.0, (int)(g() % 200) - 100);
+    printf("add %a %a %a\n", a, b, fx_double(fx_add(fx_of(a), fx_of(b))));
+  }
+  double w[6] = {1.0, NAN, 1.0, 1.0, 1.0, 1.0}, z[6] = {3.0, 3.0, 3.0, 3.0, 3.0, 3.0};
+  int2 q[6];
+  int e;
+  fx_differences<6>(w, 1.0, q, e);
+  printf("nan %a %a %a\n", fx_double(fx_value(q[0]), e - 58), fx_double(fx_add(fx_of(INFINITY), fx_of(1.0))), fx_double(fx_add(fx_of(1.0), fx_of(NAN))));
+  fx_differences<6>(z, 3.0, q, e);
+  printf("zero %a\n", fx_double(fx_value(q[2]), e - 58));
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def lines(tmp_path_factory):
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    if not os.path.exists(nvcc):
+        pytest.skip("nvcc not found")
+    d = tmp_path_factory.mktemp("fixed")
+    (d / "t.cu").write_text(PROGRAM)
+    subprocess.run([nvcc, "-O2", "-std=c++17", "-gencode", "arch=compute_103a,code=sm_103a", "-I", CSRC, "-o", str(d / "t"),
+                    str(d / "t.cu")], check=True, capture_output=True)
+    return [x.split() for x in subprocess.run([str(d / "t")], check=True, capture_output=True, text=True).stdout.splitlines()]
+
+
+def _exact(x):
+    return Fraction(float.fromhex(x))
+
+
+def test_contractions(lines):
+    n = 0
+    for w in (w for w in lines if w[0] == "sum"):
+        M, u0 = int(w[1]), _exact(w[2])
+        P, U = [_exact(x) for x in w[3:-1:2]], [_exact(x) for x in w[4:-1:2]]
+        exact = sum(p * (x - u0) for p, x in zip(P, U))
+        scale = sum(abs(p) for p in P) * max(abs(x - u0) for x in U)
+        bound = scale * (Fraction(1, 1 << 57) + M * Fraction(3, 1 << 58)) + abs(exact) / (1 << 53) + Fraction(1, 1 << 1074)
+        assert abs(_exact(w[-1]) - exact) <= bound, (M, float(abs(_exact(w[-1]) - exact) / scale))
+        n += 1
+    assert n == 40 * 3 * 4 * 3
+
+
+def test_conversions(lines):
+    for w in (w for w in lines if w[0] == "double"):
+        exact = int(w[1]) * Fraction(2) ** int(w[2])
+        if abs(exact) < Fraction(2) ** 1024:  # one rounding to nearest, or a subnormal result
+            assert abs(_exact(w[3]) - exact) <= abs(exact) / (1 << 53) + Fraction(1, 1 << 1074)
+        else:
+            assert float.fromhex(w[3]) in (float("inf"), float("-inf"))
+    for w in (w for w in lines if w[0] == "add"):
+        a, b = _exact(w[1]), _exact(w[2])
+        assert abs(_exact(w[3]) - (a + b)) <= abs(a + b) / (1 << 53) + max(abs(a), abs(b)) / (1 << 59)
+
+
+def test_special_values(lines):
+    nan = next(w for w in lines if w[0] == "nan")
+    assert all(x.strip("-") == "nan" for x in nan[1:])
+    assert float.fromhex(next(w for w in lines if w[0] == "zero")[1]) == 0.0
