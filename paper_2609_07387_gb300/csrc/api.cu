@@ -785,7 +785,7 @@ int launch_recon(ucns_mesh* m, const double* U, cudaStream_t s) {
 }
 // float pair of a caller state before a mixed reconstruction of it
 int launch_split_raw(ucns_mesh* m, const double* U, cudaStream_t s) {
-  k_split<<<nblocks((size_t)5 * m->N), 256, 0, s>>>(U, m->d.Uhl, (int)m->N);
+  k_split<<<nblocks((size_t)m->N, kSplitCells), kSplitCells, 0, s>>>(U, m->d.Uhl, (int)m->N);
   UCNS_CUDA(cudaGetLastError());
   return UCNS_OK;
 }

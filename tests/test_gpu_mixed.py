@@ -133,3 +133,18 @@ def test_float_pair_equals_its_definition():
     assert np.array_equal(hi.view(np.uint32), hi_ref.view(np.uint32))
     assert np.array_equal(lo.view(np.uint32) & 0x7fffffff, lo_ref.view(np.uint32) & 0x7fffffff)  # +-0 alike
     assert np.array_equal(lo, lo_ref)
+
+
+@pytest.mark.parametrize("n", [8, 9, 11])
+def test_split_of_the_state_equals_the_kept_pairs(n):
+    """Each single step splits the state into float pairs anew, several steps in one
+    call keep the pairs of the RK stage: the same bits on whole blocks of 128 cells
+    (8^3) and on ragged ones of 89 and 51 cells (an odd number of pairs)."""
+    nodes, cells, box = I.hex_lattice(n, jitter=0.1, seed=n)
+    m = _mesh(nodes, cells, box, 1, Mach=1.25, order=2, scheme=1)
+    a = torch.from_numpy(np.ascontiguousarray(m.to_internal(I.tgv_perturbed_state(nodes, cells, 1.25, 0.05, seed=n)))).cuda()
+    b = a.clone()
+    m.rk_steps(a, 3)
+    for _ in range(3):
+        m.rk_step(b)
+    assert torch.equal(a, b)
