@@ -155,6 +155,14 @@ __host__ __device__ __forceinline__ int2 fx_operand(double d, int eb) {
   return fx_limbs((long long)((q ^ sgn) - sgn));
 }
 
+// d shifted up by its lz - 1 spare leading bits and rounded to an operand of B bits.  The
+// shifted value may lie within a rounding unit of 2^63 (a difference just below a power
+// of two), so half a unit is added only after the shift down: |q| <= 2^B.
+template <int B>
+__host__ __device__ __forceinline__ int2 fx_normalised(long long d, int lz) {
+  return fx_limbs((((d << (lz - 1)) >> (62 - B)) + 1) >> 1);
+}
+
 // The differences u[m] - u0, m < M, as operands q[m] of one sum: all values as
 // integers aligned to the largest exponent among them, subtracted exactly, then
 // shifted up by their common leading bits.  e: |u[m] - u0| < 2^e (kFxNan when a
@@ -192,7 +200,7 @@ __host__ __device__ __forceinline__ void fx_differences(double (&u)[M], double u
   }
   const int lz = fx_clz(any | 1u);
 #pragma unroll
-  for (int m = 0; m < M; m++) q[m] = fx_limbs(((d[m] << (lz - 1)) + (1ll << (62 - B))) >> (63 - B));
+  for (int m = 0; m < M; m++) q[m] = fx_normalised<B>(d[m], lz);
   e = eb == 2047 ? kFxNan : eb - 1020 - lz - low;
 }
 

@@ -208,10 +208,7 @@ __global__ void __launch_bounds__(HOFxTile<ORDER>::THREADS, 2) k_recon_ho(ReconA
     }
     const int lz = fx_clz(any);
 #pragma unroll 4
-    for (int m = 0; m < MC; m++) {
-      const int2 w = fx_limbs(((col[m * L] << (lz - 1)) + (1ll << (62 - B))) >> (63 - B));
-      *reinterpret_cast<int2*>(&col[m * L]) = w;
-    }
+    for (int m = 0; m < MC; m++) *reinterpret_cast<int2*>(&col[m * L]) = fx_normalised<B>(col[m * L], lz);
     ec = eb == 2047 ? kFxNan : eb - 1020 - lz - (low ? 512 : 0);
   }
   const int2* op = reinterpret_cast<const int2*>(sQ) + t;

@@ -38,7 +38,44 @@ template <int M> void sums(double scale, double spread) {
     printf(" %a\n", fx_double(fx_sum(acc), E + e - 2 - fx_bits_of(M)));
   }
 }
+// one sum of edge values: members that are signed powers of two, their neighbours in
+// FP64, or of many decades, against centres far below (dir 0), or the reverse (dir 1)
+template <int M> void edge(int k, int j, int kind, int dir, double sign) {
+  double P[M], U[M], l1 = 0.0;
+  const double big = sign * std::ldexp(1.0, k), small = (j % 2 ? -1.0 : 1.0) * std::ldexp(1.0 + 0.7 * (j % 3), k - j);
+  double u0 = dir ? big : small;
+  if (kind == 1 && dir) u0 = std::nextafter(big, 0.0);
+  for (int m = 0; m < M; m++) {
+    double x = dir ? small : big;
+    if (m % 3 == 1) x = dir ? -small : small;
+    if (kind == 1 && !dir) x = m % 2 ? std::nextafter(x, 0.0) : std::nextafter(x, 2.0 * x);
+    if (kind == 2 && m % 3) x = u() * std::ldexp(1.0, k - (int)(g() % 120));
+    U[m] = x;
+    P[m] = u();
+    l1 += std::fabs(P[m]);
+  }
+  printf("edge %d %a", M, u0);
+  for (int m = 0; m < M; m++) printf(" %a %a", P[m], U[m]);
+  const int E = fx_row_exponent(l1);
+  int2 q[M];
+  int e;
+  fx_differences<M>(U, u0, q, e);
+  FxAcc acc;
+  for (int m = 0; m < M; m++) fx_mac(acc, fx_limbs(fx_round(std::ldexp(P[m], 60 - E))), q[m]);
+  printf(" %a\n", fx_double(fx_sum(acc), E + e - 2 - fx_bits_of(M)));
+}
+template <int M> void edges() {
+  for (int k : {0, 8, -3})
+    for (int j = 50; j <= 66; j++)
+      for (int kind = 0; kind < 3; kind++)
+        for (int dir = 0; dir < 2; dir++)
+          for (double sign : {1.0, -1.0}) edge<M>(k, j, kind, dir, sign);
+}
 int main() {
+  edges<6>();
+  edges<18>();
+  edges<38>();
+  edges<68>();
   for (double spread : {1e-9, 0.1, 10.0})
     for (double scale : {1.0, 1e-200, 1e200, 0x1p-1000}) { sums<6>(scale, spread); sums<18>(scale, spread); sums<68>(scale, spread); }
   for (int t = 0; t < 4000; t++) {
@@ -86,6 +123,24 @@ def test_contractions(lines):
         assert abs(_exact(w[-1]) - exact) <= bound, (M, float(abs(_exact(w[-1]) - exact) / scale))
         n += 1
     assert n == 40 * 3 * 4 * 3
+
+
+def _check(w):
+    M, u0 = int(w[1]), _exact(w[2])
+    P, U = [_exact(x) for x in w[3:-1:2]], [_exact(x) for x in w[4:-1:2]]
+    exact = sum(p * (x - u0) for p, x in zip(P, U))
+    scale = sum(abs(p) for p in P) * max(abs(x - u0) for x in U)
+    bound = scale * (Fraction(1, 1 << 57) + M * Fraction(3, 1 << 58)) + abs(exact) / (1 << 53)
+    return M, w[2], float(abs(_exact(w[-1]) - exact) / scale) if abs(_exact(w[-1]) - exact) > bound else 0.0
+
+
+def test_contractions_at_powers_of_two(lines):
+    """Differences within a few units of a power of two: members that are signed powers
+    of two (or next to one, or spread over 120 binades) and centres 2^-50 to 2^-66 of
+    them, either way round, in the header's bound (test_contractions states it)."""
+    off = [_check(w) for w in lines if w[0] == "edge"]
+    assert len(off) == 4 * 3 * 17 * 3 * 2 * 2
+    assert [x for x in off if x[2]] == []
 
 
 def test_conversions(lines):

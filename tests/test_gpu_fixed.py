@@ -82,6 +82,24 @@ def test_power_of_two_states_scale_exactly(order, k):
     assert np.array_equal(_residual(m, U * 2.0 ** k), _residual(m, U) * 2.0 ** k)
 
 
+# Exact units beside round-off: differences just below a power of two, which round up
+# to it (both signs, central and directional stencils)
+@pytest.mark.parametrize("scheme", [0, 1])
+@pytest.mark.parametrize("order", [2, 3, 4])
+def test_units_beside_round_off(order, scheme):
+    m, oc, U = _both("hexes", (9, 9, 10), order, scheme, mach=1.0)
+    rng = np.random.default_rng(8)
+    unit, tiny = rng.random(U.shape[1]) < 0.5, rng.choice([1e-18, -1e-18, 3e-18, -2e-19], size=U.shape[1])
+    U[0], U[4] = 1.0, 10.0
+    U[1] = np.where(unit, 1.0, tiny)
+    U[2] = np.where(unit, -1.0, tiny)
+    U[3] = np.where(unit, tiny, 0.5)
+    R, (Rc, S) = _residual(m, U), oc.residual_terms(U)
+    err = np.abs(R - Rc).max(axis=1) / S.max(axis=1)
+    print(order, scheme, err)
+    assert np.all(err <= 1e-12)
+
+
 @pytest.mark.parametrize("order", [2, 3, 4])
 @pytest.mark.parametrize("bad", [np.nan, np.inf])
 def test_non_finite_states_stay_visible(order, bad):
