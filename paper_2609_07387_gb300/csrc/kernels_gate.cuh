@@ -118,16 +118,17 @@ __global__ void __launch_bounds__(128) k_features(FeatArgs a) {
 #pragma unroll
     for (int k = 0; k < K; k++) {
       const int2 q = __ldg(&P[(k * MC + m) * FxTile::TC]);
-      // 2^60 P_km 2^-E_k from the limbs, its upper 23 bits exact and the others in one
-      // conversion each; the row's scale follows after the sum
-      const float p = fmaf((float)(q.x >> 8), 0x1p38f, (float)(((q.x & 0xff) << 22) + (q.y >> 8)) * 0x1p8f);
+      // P_km 2^-E_k (below one, so that the sums overflow no earlier than the coefficients)
+      // from the limbs, its upper 23 bits exact and the others in one conversion each; the
+      // row's scale follows after the sum
+      const float p = fmaf((float)(q.x >> 8), 0x1p-22f, (float)(((q.x & 0xff) << 22) + (q.y >> 8)) * 0x1p-52f);
 #pragma unroll
       for (int v = 0; v < 5; v++) ao[v][k] = fmaf(p, d[v], ao[v][k]);
     }
   }
 #pragma unroll
   for (int k = 0; k < K; k++) {
-    const int e = (int)__ldg(&E[k * FxTile::TC]) - 60;
+    const int e = (int)__ldg(&E[k * FxTile::TC]);
 #pragma unroll
     for (int v = 0; v < 5; v++) ao[v][k] = ldexpf(ao[v][k], e);
   }

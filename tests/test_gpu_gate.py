@@ -162,6 +162,21 @@ def test_features_and_labels_match_oracle(prec):
     assert np.abs(dev - odev).max() <= 1e-6
 
 
+@pytest.mark.parametrize("k", [90, -90])
+def test_features_of_scaled_states(k):
+    """FP64 form: the features that are ratios of equal powers of the state (differences,
+    Mach number, divergence, vorticity) do not change with its scale 2^k while the FP32
+    coefficients are in range; every operation on them scales exactly.  The smoothness
+    ratios 24-28 square the coefficients and overflow at this scale by themselves."""
+    nodes, cells, box = I.hex_lattice(9, jitter=0.1, seed=4)
+    m = ucns.Mesh(nodes, cells, box, ucns.Params(order=2, scheme=1, Mach=1.25))
+    U = m.to_internal(I.tgv_perturbed_state(nodes, cells, 1.25, 0.05, seed=4))
+    F = [m.gate_features(torch.from_numpy(np.ascontiguousarray(U * s)).cuda(), want_f32=True)[1].cpu().numpy()
+         for s in (1.0, 2.0 ** k)]
+    ratios = np.r_[0:24, 29:32]
+    assert np.all(np.isfinite(F[0])) and np.array_equal(F[0][:, ratios], F[1][:, ratios])
+
+
 @pytest.mark.parametrize("tets", [False, True])
 def test_gated_residual_extremes_equal_the_plain_schemes(tets):
     """Hexahedra (6 directional stencils) and tetrahedra (4): a gate that flags
