@@ -151,8 +151,8 @@ int ucns_mesh_set_boundary(ucns_mesh* mesh, const int32_t* kinds, const double* 
  * built in the FP64 form at P1 and P2.  Device memory is dominated by the
  * pseudo-inverses: per cell about 2.7 KB (P2 FP64 CWENOZ), 10 / 36 KB (P3 / P4
  * FP64) and 4.4 / 16.2 KB (P3 / P4 mixed, held in 32-cell tile records); the
- * host needs the FP64 arrays and, briefly, the device layout's copy.  Errors:
- * INVALID_ARG, STENCIL, CUDA, NOMEM (also when the host runs out of memory
+ * host needs the FP64 arrays and, briefly, the device layout's copy (mixed
+ * form) or pieces of it of 64 MB (FP64 form).  Errors: INVALID_ARG, STENCIL, CUDA, NOMEM (also when the host runs out of memory
  * while building the device arrays; nothing stays allocated). */
 int ucns_precompute(ucns_mesh* mesh, const ucns_params* params);
 

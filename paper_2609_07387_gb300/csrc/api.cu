@@ -75,46 +75,85 @@ int upload_blocked(T** dst, const std::vector<S>& src, int rows, int64_t N, bool
   return upload(dst, b);
 }
 
+template <typename T>
+int alloc(T** dst, size_t n) {
+  if (cudaMalloc((void**)dst, n * sizeof(T)) != cudaSuccess)
+    return fail(UCNS_ERR_NOMEM, "cudaMalloc failed for library scratch");
+  return UCNS_OK;
+}
+
+// Tile records are converted and copied in pieces of this many bytes of host memory: the
+// rows that they come from stay alive beside them, and all records together are as large
+// (2.4 / 10 / 36 KB a cell at P2 / P3 / P4).
+constexpr int64_t kPieceBytes = 64 << 20;
+inline int64_t tiles_in_piece(int64_t tiles, int rec) { return std::min(tiles, std::max<int64_t>(1, kPieceBytes / rec)); }
+
 // the P2 reconstruction's tiles (FxTile) of the FP64 form
 int upload_fx_tiles(const ucns_mesh* m, const HostArrays& h, unsigned char** dst) {
   const int rec = FxTile::record(m->nd);
-  const int64_t tiles = (m->N + FxTile::TC - 1) / FxTile::TC;
-  std::vector<unsigned char> b((size_t)tiles * rec, 0);
+  const int64_t tiles = (m->N + FxTile::TC - 1) / FxTile::TC, step = tiles_in_piece(tiles, rec);
+  int rc = alloc(dst, (size_t)tiles * rec);
+  if (rc) return rc;
+  std::vector<unsigned char> b((size_t)step * rec);
+  for (int64_t t0 = 0; t0 < tiles; t0 += step) {
+    const int64_t n = std::min(step, tiles - t0);
 #pragma omp parallel for schedule(static)
-  for (int64_t t = 0; t < tiles; t++) fx_tile(h, m->nd, m->N, t, b.data() + (size_t)t * rec);
-  return upload(dst, b);
+    for (int64_t t = 0; t < n; t++) {
+      unsigned char* r = b.data() + (size_t)t * rec;
+      std::memset(r, 0, rec);
+      fx_tile(h, m->nd, m->N, t0 + t, r);
+    }
+    UCNS_CUDA(cudaMemcpy(*dst + (size_t)t0 * rec, b.data(), (size_t)n * rec, cudaMemcpyHostToDevice));
+  }
+  return UCNS_OK;
 }
 
 // the smoothness-indicator matrices' leading Kd x Kd block, upper triangle by rows
-std::vector<double> leading_block(const ucns_mesh* m, const HostArrays& h) {
+int upload_leading_block(const ucns_mesh* m, const HostArrays& h, double** dst) {
+  if (h.Msi.empty()) return UCNS_OK;
   const int K = m->K, Kd = m->Kd;
-  const int64_t N = m->N;
-  std::vector<double> b;
-  b.reserve((size_t)Kd * (Kd + 1) / 2 * N);
+  const size_t N = m->N;
+  int rc = alloc(dst, Kd * (Kd + 1) / 2 * N);
+  if (rc) return rc;
+  double* at = *dst;
   for (int k = 0; k < Kd; k++) {
-    const auto row = h.Msi.begin() + (size_t)(k * K - k * (k - 1) / 2) * N;
-    b.insert(b.end(), row, row + (size_t)(Kd - k) * N);
+    const size_t n = (Kd - k) * N;
+    UCNS_CUDA(cudaMemcpy(at, h.Msi.data() + (k * K - k * (k - 1) / 2) * N, n * sizeof(double), cudaMemcpyHostToDevice));
+    at += n;
   }
-  return b;
+  return UCNS_OK;
 }
 
 // the P3/P4 reconstruction's tiles (HOFxTile) of the FP64 form, their stencils and row exponents
 template <int ORDER>
 int upload_ho_fx_tiles(const ucns_mesh* m, const HostArrays& h, DeviceMesh& d) {
   using T = HOFxTile<ORDER>;
+  constexpr size_t IDS = T::IDS * T::TC, EXPS = T::EXPS * T::TC;  // entries per tile
   const bool weno = m->nd > 0;
-  const int64_t tiles = (m->N + T::TC - 1) / T::TC;
   const int rec = T::record(weno);
-  std::vector<unsigned char> b((size_t)tiles * rec, 0);
-  std::vector<int32_t> ids((size_t)tiles * T::IDS * T::TC, 0);
-  std::vector<int16_t> exps((size_t)tiles * T::EXPS * T::TC, 0);
+  const int64_t tiles = (m->N + T::TC - 1) / T::TC, step = tiles_in_piece(tiles, rec);
+  int rc;
+  if ((rc = alloc(&d.fxt, (size_t)tiles * rec)) || (rc = alloc(&d.fx_ids, tiles * IDS)) ||
+      (rc = alloc(&d.fx_exps, tiles * EXPS)))
+    return rc;
+  std::vector<unsigned char> b((size_t)step * rec);
+  std::vector<int32_t> ids(step * IDS);
+  std::vector<int16_t> exps(step * EXPS);
+  for (int64_t t0 = 0; t0 < tiles; t0 += step) {
+    const int64_t n = std::min(step, tiles - t0);
 #pragma omp parallel for schedule(static)
-  for (int64_t t = 0; t < tiles; t++)
-    ho_fx_tile<ORDER>(h, weno, m->N, t, b.data() + (size_t)t * rec, &ids[(size_t)t * T::IDS * T::TC],
-                      &exps[(size_t)t * T::EXPS * T::TC]);
-  int rc = upload(&d.fxt, b);
-  if (rc || (rc = upload(&d.fx_ids, ids))) return rc;
-  return upload(&d.fx_exps, exps);
+    for (int64_t t = 0; t < n; t++) {
+      unsigned char* r = b.data() + (size_t)t * rec;
+      std::memset(r, 0, rec);
+      std::fill_n(&ids[t * IDS], IDS, 0);
+      std::fill_n(&exps[t * EXPS], EXPS, (int16_t)0);
+      ho_fx_tile<ORDER>(h, weno, m->N, t0 + t, r, &ids[t * IDS], &exps[t * EXPS]);
+    }
+    UCNS_CUDA(cudaMemcpy(d.fxt + (size_t)t0 * rec, b.data(), (size_t)n * rec, cudaMemcpyHostToDevice));
+    UCNS_CUDA(cudaMemcpy(d.fx_ids + t0 * IDS, ids.data(), n * IDS * sizeof(int32_t), cudaMemcpyHostToDevice));
+    UCNS_CUDA(cudaMemcpy(d.fx_exps + t0 * EXPS, exps.data(), n * EXPS * sizeof(int16_t), cudaMemcpyHostToDevice));
+  }
+  return UCNS_OK;
 }
 
 // The FP64 face geometry from P2 on: per cell the exponents of its axis scales (the
@@ -148,13 +187,6 @@ int upload_fixed_faces(const ucns_mesh* m, double** dst, int16_t** dst_h, std::v
     }
   int rc = upload(dst, fq);
   return rc ? rc : upload(dst_h, h);
-}
-
-template <typename T>
-int alloc(T** dst, size_t n) {
-  if (cudaMalloc((void**)dst, n * sizeof(T)) != cudaSuccess)
-    return fail(UCNS_ERR_NOMEM, "cudaMalloc failed for library scratch");
-  return UCNS_OK;
 }
 
 inline unsigned nblocks(size_t threads, int bs = 256) { return (unsigned)((threads + bs - 1) / bs); }
@@ -1213,7 +1245,7 @@ static int device_upload(ucns_mesh* m, const ucns_params* p, HostArrays& h) {
              (m->K == 3 && (rc = upload(&d.fq, h.fq))) ||
              (m->K > 3 && ((rc = upload_fixed_faces(m, &d.fq, &d.hexp, h.fq)) ||
                             (rc = alloc(&d.cexp, (size_t)5 * m->N)))) ||
-             (rc = upload(&d.fpen, h.fpen)) || (m->K > 9 && (rc = upload(&d.Msi, leading_block(m, h)))) ||
+             (rc = upload(&d.fpen, h.fpen)) || (m->K > 9 && (rc = upload_leading_block(m, h, &d.Msi))) ||
              (rc = upload(&d.psib, h.psib)) ||
              (rc = alloc(&d.coef, (size_t)m->NC * m->N * 5))) {
     device_free(m);

@@ -3,6 +3,10 @@ wrong: ragged tiles of every element kind, weights whose common denominator
 leaves the product range, states whose differences are subnormal before they
 are aligned, and non-finite states; against the oracle at its FP64 bar (1e-12
 of the summed-term scale, tests/test_gpu_parity.py)."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -106,3 +110,27 @@ def test_non_finite_states_stay_visible(order, bad):
     m, oc, U = _both("hexes", (11, 11, 12), order, 0)
     U[1, 700] = bad
     assert np.array_equal(np.isfinite(_residual(m, U)), np.isfinite(oc.residual(U)))
+
+
+# The FP64 form's tiles (35 KB a cell at P4, like the rows they are converted from) are
+# uploaded in pieces: building a mesh takes the rows and little more of host memory
+def test_host_memory_while_a_mesh_is_built():
+    code = """
+import numpy as np
+from paper_2609_07387_gb300 import inputs as I, ucns
+def peak():
+    return next(int(x.split()[1]) for x in open("/proc/self/status") if x.startswith("VmHWM")) * 1024
+def build(n):
+    nodes, cells, box = I.hex_lattice(n, jitter=0.1, seed=5)
+    return ucns.Mesh(nodes, cells, box, ucns.Params(order=4, scheme=1))
+small = build(9)  # the CUDA context and the modules
+before = peak()
+build(24)
+print(peak() - before)
+"""
+    out = subprocess.run([sys.executable, "-c", code], check=True, capture_output=True, text=True, timeout=300,
+                         cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__)))).stdout
+    # rows, matrices, stencils and face points in FP64
+    rows = 24 ** 3 * (8 * (34 * 68 + 6 * 9 * 18 + 595 + 31) + 4 * (68 + 108) + 3 * 8 * 160)
+    print(int(out) / rows)
+    assert int(out) < 1.5 * rows
