@@ -47,9 +47,15 @@ __host__ __device__ __forceinline__ int2 fx_limbs(long long q) {
 // x rounded to an integer (host; |x| < 2^62, exact from 2^53 on)
 inline long long fx_round(double x) { return (long long)(x + std::copysign(0.5, x)); }
 
-// exponent E of a row: sum |P_m| < 2^E (a row of zeros: 0)
+// An exponent of kFxNan or a little below makes fx_double a NaN (a non-finite operand
+// or row).  Exponents of finite sums stay below 2^13: operands and rows below 2^11
+// each, and axis scales, of cells whose volume and its square are finite, below 2^10.
+constexpr int kFxNan = 1 << 15;
+
+// exponent E of a row: sum |P_m| < 2^E (a row of zeros: 0; with a NaN or an infinity: kFxNan - 1)
 inline int fx_row_exponent(double l1) {
   int e = 0;
+  if (!std::isfinite(l1)) return kFxNan - 1;
   if (l1 > 0.0) std::frexp(l1, &e);
   return e;
 }
@@ -78,8 +84,6 @@ __host__ __device__ __forceinline__ void fx_mac(FxAcc& a, int2 p, int2 d) {
 __host__ __device__ __forceinline__ long long fx_sum(const FxAcc& a) {
   return (a.h << 2) + ((a.m + (1ll << 27)) >> 28);
 }
-
-constexpr int kFxNan = 1 << 20;  // an exponent that makes fx_double a NaN (a non-finite operand)
 
 __host__ __device__ __noinline__ static double fx_double_rare(long long s, int e) {
   if (e >= kFxNan / 2) return (double)NAN;

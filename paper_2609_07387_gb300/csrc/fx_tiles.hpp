@@ -15,7 +15,8 @@
 namespace ucns {
 
 // One matrix row of nc <= 32 consecutive cells, entry m of cell c at row(m)[c], as
-// limb pairs at(m)[c] and exponents E[c] (fixed.cuh)
+// limb pairs at(m)[c] and exponents E[c] (fixed.cuh); a row with a NaN or an infinity
+// (a smoothness matrix whose moments left FP64's range) has zeros and the NaN exponent
 template <class Row, class At>
 void fixed_row(const Row& row, int M, int nc, const At& at, int16_t* E) {
   double l1[32] = {0.0}, up[32], more[32];
@@ -32,7 +33,7 @@ void fixed_row(const Row& row, int M, int nc, const At& at, int16_t* E) {
   for (int m = 0; m < M; m++) {
     const double* x = row(m);
     int2* q = at(m);
-    for (int c = 0; c < nc; c++) q[c] = fx_limbs(fx_round(x[c] * up[c] * more[c]));
+    for (int c = 0; c < nc; c++) q[c] = E[c] == kFxNan - 1 ? make_int2(0, 0) : fx_limbs(fx_round(x[c] * up[c] * more[c]));
   }
 }
 

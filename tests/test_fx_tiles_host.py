@@ -124,20 +124,54 @@ template <int ORDER> int ho() {
   return bad;
 }
 
+// a sum over a row of two cells, the second's with one entry bad, times members 1, ..., 6
+void non_finite(double bad) {
+  double x[6][2], U[6];
+  int2 P[6][2], q[6];
+  int16_t E[2];
+  int e;
+  for (int m = 0; m < 6; m++) {
+    x[m][0] = x[m][1] = 0.25 * m;
+    U[m] = 1.0 + m;
+  }
+  x[4][1] = bad;
+  fixed_row([&](int m) { return x[m]; }, 6, 2, [&](int m) { return P[m]; }, E);
+  fx_differences<6>(U, 0.0, q, e);
+  for (int c = 0; c < 2; c++) {
+    FxAcc acc;
+    for (int m = 0; m < 6; m++) fx_mac(acc, P[m][c], q[m]);
+    printf(" %g", fx_double(fx_sum(acc), E[c] + e - 2 - fx_bits_of(6)));
+  }
+}
+
 int main() {
   const int a = p2(0) + p2(6), b = ho<3>(), c = ho<4>();
-  printf("%d %d %d %d\n", a, b, c, (int)allocations);
+  printf("%d %d %d %d", a, b, c, (int)allocations);
+  non_finite(NAN);
+  non_finite(INFINITY);
+  non_finite(-INFINITY);
+  printf("\n");
 }
 """
 
 
-def test_tiles(tmp_path):
+@pytest.fixture(scope="module")
+def out(tmp_path_factory):
     nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
     if not os.path.exists(nvcc):
         pytest.skip("nvcc not found")
-    (tmp_path / "t.cu").write_text(PROGRAM)
-    subprocess.run([nvcc, "-O1", "-std=c++17", "-gencode", "arch=compute_103a,code=sm_103a", "-I", CSRC, "-o", str(tmp_path / "t"),
-                    str(tmp_path / "t.cu")], check=True, capture_output=True)
-    out = subprocess.run([str(tmp_path / "t")], check=True, capture_output=True, text=True).stdout.split()
+    d = tmp_path_factory.mktemp("tiles")
+    (d / "t.cu").write_text(PROGRAM)
+    subprocess.run([nvcc, "-O1", "-std=c++17", "-gencode", "arch=compute_103a,code=sm_103a", "-I", CSRC, "-o", str(d / "t"),
+                    str(d / "t.cu")], check=True, capture_output=True)
+    return subprocess.run([str(d / "t")], check=True, capture_output=True, text=True).stdout.split()
+
+
+def test_tiles(out):
     assert out[:3] == ["0", "0", "0"]  # misplaced entries at P2, P3, P4
     assert out[3] == "0"  # allocations while a tile is converted
+
+
+def test_non_finite_rows_give_nan(out):
+    """As FP64 sums do: 17.5 over the sound row, NaN over one with a NaN or an infinity."""
+    assert [x.strip("-") for x in out[4:]] == ["17.5", "nan"] * 3
