@@ -146,14 +146,14 @@ __host__ __device__ __forceinline__ long long fx_integer(double x, int eb) {
   return (long long)((q ^ sgn) - sgn);
 }
 
-// operand q of d, rounded to B bits, for a sum whose largest biased exponent is
-// eb (64 <= eb < 2047, or every d zero)
+// operand q of d, rounded to B bits, for a sum whose largest biased exponent is eb < 2047
+// (d normal and at most that large, zero, or subnormal and eb at least 64)
 template <int B>
 __host__ __device__ __forceinline__ int2 fx_operand(double d, int eb) {
   const unsigned long long b = fx_bits(d);
   const int e = (int)((unsigned)(b >> 52) & 0x7ffu);
   const unsigned long long mant = (b & 0xfffffffffffffull) | ((unsigned long long)(e != 0) << 52);
-  const int sh = eb - e < 63 ? eb - e : 63;
+  const unsigned sh = (unsigned)(eb - e) < 63u ? (unsigned)(eb - e) : 63u;
   const unsigned long long q = (((mant << (B - 52)) >> sh) + 1) >> 1;
   const unsigned long long sgn = (unsigned long long)((long long)b >> 63);
   return fx_limbs((long long)((q ^ sgn) - sgn));
@@ -208,29 +208,48 @@ __host__ __device__ __forceinline__ void fx_differences(double (&u)[M], double u
   e = eb == 2047 ? kFxNan : eb - 1020 - lz - low;
 }
 
-// The same for polynomial coefficients d[k], each to be scaled by 2^off[k].
+// The same for polynomial coefficients d[k], each to be scaled by 2^off[k]: returns eb,
+// from which fx_operand(d[k], eb - off[k]) are the operands of exponent e.  Zeros take no
+// part (the offset of one may lie far above the others); subnormal coefficients, which
+// with a large offset need not be small, are made normal first (exact), unless one
+// beside them is so large that they do not count.
 template <int M>
 __host__ __device__ __forceinline__ int fx_align_scaled(double (&d)[M], const int (&off)[M], int& e) {
-  bool bad = false;
-  int eb = -(1 << 14);
+  constexpr int none = -(1 << 14);
+  int eb = none;
+  bool odd = false;  // a zero, subnormal or non-finite coefficient
 #pragma unroll
   for (int m = 0; m < M; m++) {
     const int x = fx_exponent(d[m]);
-    bad = bad || x == 2047;
+    odd = odd || (unsigned)(x - 1) >= 2046u;
     eb = x + off[m] > eb ? x + off[m] : eb;
   }
   e = eb - 1022;
-  if (eb < 64) {
-    eb = -(1 << 14);
+  if (odd) {
+    auto largest = [&](bool& sub, int& top) {
+      int r = none;
 #pragma unroll
-    for (int m = 0; m < M; m++) {
-      d[m] *= 0x1p512;
-      const int x = fx_exponent(d[m]);
-      eb = x + off[m] > eb ? x + off[m] : eb;
+      for (int m = 0; m < M; m++) {
+        const int x = fx_exponent(d[m]);
+        if (fx_bits(d[m]) << 1 == 0ull) continue;
+        sub = sub || x == 0;
+        top = x > top ? x : top;
+        r = x + off[m] > r ? x + off[m] : r;
+      }
+      return r;
+    };
+    bool sub = false;
+    int top = 0;
+    eb = largest(sub, top);
+    e = eb - 1022;
+    if (sub && top < 1500) {
+#pragma unroll
+      for (int m = 0; m < M; m++) d[m] *= 0x1p512;
+      eb = largest(sub, top);
+      e = eb - 1022 - 512;
     }
-    e = eb - 1022 - 512;
+    if (top == 2047) e = kFxNan;
   }
-  if (bad) e = kFxNan;
   return eb;
 }
 

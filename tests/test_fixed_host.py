@@ -13,6 +13,7 @@ import pytest
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2609_07387_gb300", "csrc")
 
 PROGRAM = r"""
+#include "basis.hpp"
 #include "fixed.cuh"
 #include <cstdio>
 #include <random>
@@ -71,7 +72,33 @@ template <int M> void edges() {
         for (int dir = 0; dir < 2; dir++)
           for (double sign : {1.0, -1.0}) edge<M>(k, j, kind, dir, sign);
 }
+// the coefficients of a polynomial on a cell of axis scale 2^h: about 2^u each in scaled
+// coordinates, so of 2^(u - deg h), some zero
+template <int ORDER> void coefficients(int h, int u2, bool zeros) {
+  constexpr int K = basis_count(ORDER), B = ORDER == 4 ? 57 : 58;
+  double c[K];
+  int off[K], e;
+  for (int k = 0; k < K; k++) {
+    off[k] = basis_degree(k) * h;
+    c[k] = std::ldexp(u(), u2 - off[k] - (int)(g() % 12));
+    if (zeros && (k >= 3 || g() % 2)) c[k] = 0.0;
+    if (!std::isfinite(c[k])) return;
+  }
+  double in[K];
+  for (int k = 0; k < K; k++) in[k] = c[k];
+  const int eb = fx_align_scaled<K>(c, off, e);
+  printf("poly %d %d", B, e);
+  for (int k = 0; k < K; k++) printf(" %a %d %lld", in[k], off[k], fx_value(fx_operand<B>(c[k], eb - off[k])));
+  printf("\n");
+}
 int main() {
+  for (int h : {-180, -20, 0, 12, 40, 90, 170})
+    for (int u2 : {0, 300, -330, -700, -860, -960, -1030})
+      for (int t = 0; t < 8; t++) {
+        coefficients<2>(h, u2, t % 2);
+        coefficients<3>(h, u2, t % 2);
+        coefficients<4>(h, u2, t % 2);
+      }
   edges<6>();
   edges<18>();
   edges<38>();
@@ -141,6 +168,27 @@ def test_contractions_at_powers_of_two(lines):
     off = [_check(w) for w in lines if w[0] == "edge"]
     assert len(off) == 4 * 3 * 17 * 3 * 2 * 2
     assert [x for x in off if x[2]] == []
+
+
+def test_coefficients(lines):
+    """Polynomial coefficients c_k scaled by 2^off_k and aligned to the largest of them
+    (csrc/kernels.cuh, store_fixed): half a unit 2^(e - B) of error each, the unit not more
+    than that of the largest; cells of any size, states that make some coefficients
+    subnormal or zero."""
+    n = 0
+    for w in (w for w in lines if w[0] == "poly"):
+        B, e = int(w[1]), int(w[2])
+        exact = [_exact(c) * Fraction(2) ** int(off) for c, off in zip(w[3::3], w[4::3])]
+        q = [int(x) for x in w[5::3]]
+        big = max(abs(x) for x in exact)
+        if big == 0:
+            assert q == [0] * len(q)
+            continue
+        unit = Fraction(2) ** (e - B)
+        assert unit <= 2 * big / (1 << B), (e, float(big))
+        assert all(abs(x - y * unit) <= unit / 2 and abs(y) <= 1 << B for x, y in zip(exact, q)), (w[:3], float(big))
+        n += 1
+    assert n > 800
 
 
 def test_conversions(lines):

@@ -86,6 +86,22 @@ def test_power_of_two_states_scale_exactly(order, k):
     assert np.array_equal(_residual(m, U * 2.0 ** k), _residual(m, U) * 2.0 ** k)
 
 
+# Cells of 2^40 with states of 2^-860: at P4 the quartic coefficients are subnormal (47
+# bits of FP64's 53 left) and the zero ones have large offsets; the residual is the
+# unit mesh's scaled, to the rounding of sums 1e3 times as large
+@pytest.mark.parametrize("order", [2, 3, 4])
+def test_large_cells_with_small_states(order):
+    nodes, cells, box = I.hex_lattice((9, 9, 10), jitter=0.1, seed=5)
+    U = I.noisy_state(nodes, cells, 1.0, 0.05, seed=6)
+    R = []
+    for L, u in ((0, 0), (40, -860)):
+        m = ucns.Mesh(nodes * 2.0 ** L, cells, np.array(box) * 2.0 ** L, ucns.Params(order=order, scheme=0, Re=0.0, Mach=1.0))
+        R.append(_residual(m, U * 2.0 ** u) * 2.0 ** (L - u))
+    err = np.abs(R[1] - R[0]).max(axis=1) / np.abs(R[0]).max(axis=1)
+    print(order, err)
+    assert np.all(err <= 1e-12)
+
+
 # Exact units beside round-off: differences just below a power of two, which round up
 # to it (both signs, central and directional stencils)
 @pytest.mark.parametrize("scheme", [0, 1])
