@@ -54,12 +54,16 @@ STAGES = 3
 ERROR_BOUND = 1e-4  # relative, on the kinetic-energy and dissipation histories
 
 # Algorithmic flop counts of the kernels (each +,-,*,/,sqrt = 1, FMA = 2), counted
-# from the kernel source.  Face kernel, per Gauss point: 2 sides x 5 variables x 33
-# (value 9 FMA, gradient 6 FMA + 3 mul) = 330, penalty and averages 80, HLLC 138,
-# viscous flux 120, scaling and the Gauss sum 20.  Reconstruction, per cell: 5 x 814
-# (central differences + contraction 342, directional 252, smoothness indicators 95,
-# weights and combination 125); linear weights only: 5 x 354.
-FLOPS_FACE_P2_VISC_PER_QP = 688
+# from the kernel source.  Face kernels, per Gauss point: values and gradients of 2 sides
+# x 5 variables in nested form (15 FMAs at P2, 35 at P3, 65 at P4) and the 15 sums of the
+# two gradients; HLLC 109, viscous flux 113, penalty, averages and difference 19, scaling
+# and the Gauss sum 10, as the FP64 form has them (the mixed form's reference-relative
+# fluxes take 31 more for the same result).  Reconstruction, per cell: 5 x 814 (central
+# differences + contraction 342, directional 252, smoothness indicators 95, weights and
+# combination 125); linear weights only: 5 x 354.
+FMAS_EVAL = {9: 15, 19: 35, 34: 65}  # by modes K
+FLOPS_FLUX_PER_QP = 109 + 113 + 19 + 10
+FLOPS_FACE_P2_VISC_PER_QP = 2 * 5 * 2 * FMAS_EVAL[9] + 15 + FLOPS_FLUX_PER_QP
 FLOPS_RECON_P2_CWENOZ_PER_CELL = 4070
 FLOPS_RECON_P2_LINEAR_PER_CELL = 5 * 354
 
@@ -323,8 +327,10 @@ def run_reference(args, cfg: Config, n: int, rank: int, world: int):
 # ------------------------------------------------------------- GPU arm
 def algorithmic(m, kind: str, mixed: bool, frac_dir: float = 1.0) -> dict:
     """Flops and bytes of one launch of the face or reconstruction kernel.
-    flops: as counted above.  bytes: each array element the kernel needs
-    crossing HBM once (neighbour gathers served by cache), in two countings:
+    flops: as counted above; pipe_flops: those on the pipe that the roofline
+    compares them with (in the FP64 form from P2 on the contractions, the P3/P4
+    smoothness rows and the polynomial evaluations run on the integer pipe).
+    bytes: each array element the kernel needs crossing HBM once (neighbour gathers served by cache), in two countings:
       "alg": the minimal data -- per Gauss point its position relative to the
         owner's centroid and its area vector (6 words), per face the offset
         between the two centroids (3 words), the penalty factor, two cell ids
@@ -345,6 +351,7 @@ def algorithmic(m, kind: str, mixed: bool, frac_dir: float = 1.0) -> dict:
     fx = 1 if m.K == 9 and not mixed else 0
     if kind == "face":
         flops = FLOPS_FACE_P2_VISC_PER_QP * nq * F
+        pipe = FLOPS_FLUX_PER_QP * nq * F if fx else flops
         face_common = 4 + 2 * 4 + 5 * w            # penalty (FP32 in both forms' count), ids, totals
         alg = F * (nq * 6 * w + 3 * w + face_common) + N * coef
         row = (((m.K + 1) * 5 + 3) // 4 * 4) * 4 if mixed else coef + fx * 28
@@ -353,6 +360,7 @@ def algorithmic(m, kind: str, mixed: bool, frac_dir: float = 1.0) -> dict:
         lin = FLOPS_RECON_P2_LINEAR_PER_CELL if m.K == 9 else 5 * 2 * m.K * m.Mc
         cw = FLOPS_RECON_P2_CWENOZ_PER_CELL if m.nd else lin
         flops = N * (lin + frac_dir * (cw - lin))
+        pipe = N * 5 * (12 + frac_dir * (208 if m.nd else 0)) if fx else flops
         cell = 7 * w                                 # six second moments and 1/h
         state = 5 * 8                                # the FP64 state, or its float pair
         base = m.K * m.Mc * w + m.Mc * 4 + cell + state
@@ -360,42 +368,36 @@ def algorithmic(m, kind: str, mixed: bool, frac_dir: float = 1.0) -> dict:
         alg = N * (base + coef + frac_dir * dirb)
         row = (((m.K + 1) * 5 + 3) // 4 * 4) * 4 if mixed else coef + fx * (28 + 2 * (m.K + 3 * m.nd))
         layout = N * (base + row + frac_dir * dirb)
-    return {"flops": flops, "alg": alg, "layout": layout}
-
-
-# exponents of the basis monomials beyond P2 (the kernels' order), for the P3/P4 flop counts
-_BASIS_HO = [(3, 0, 0), (2, 1, 0), (2, 0, 1), (1, 2, 0), (1, 1, 1), (1, 0, 2), (0, 3, 0), (0, 2, 1), (0, 1, 2),
-             (0, 0, 3), (4, 0, 0), (3, 1, 0), (3, 0, 1), (2, 2, 0), (2, 1, 1), (2, 0, 2), (1, 3, 0), (1, 2, 1),
-             (1, 1, 2), (1, 0, 3), (0, 4, 0), (0, 3, 1), (0, 2, 2), (0, 1, 3), (0, 0, 4)]
-_BASIS_P2 = [(1, 0, 0), (0, 1, 0), (0, 0, 1), (2, 0, 0), (0, 2, 0), (0, 0, 2), (1, 1, 0), (1, 0, 1), (0, 1, 1)]
+    return {"flops": flops, "pipe_flops": pipe, "alg": alg, "layout": layout}
 
 
 def algorithmic_ho(m, kind: str, w: int = 8) -> dict:
     """Flops and bytes of one launch of the P3/P4 kernels (w: bytes per word,
     8 in the FP64 form, 4 in the mixed one; ids 4, the state 8), counted
-    from their source: face, per Gauss point, 2 sides x 5 variables x 2 flops
-    x (K value terms + one gradient term per nonzero exponent), the
-    monomials' products (4 per mode and side), HLLC 138, viscous 120,
-    penalty/averages 80, scaling and sum 20; reconstruction, per cell, the
-    central contraction and differences, the directional contractions twice,
-    the smoothness forms (K^2 central, Kd^2 per candidate) and the weights."""
-    basis = (_BASIS_P2 + _BASIS_HO)[:m.K]
+    from their source: face as above; reconstruction, per cell and variable,
+    the central differences and contraction, with CWENOZ the directional ones
+    (once: the candidates are kept), the smoothness forms (K^2 central, Kd^2
+    per candidate; the FP64 form's central rows are integer sums, 2 K flops
+    are left) and the weights (60), and the scaling (2 K)."""
     N, F, nq, K = m.n_cells, m.n_faces, m.nq, m.K
     kd = m.Md // 2
     if kind == "face":
-        g = sum(sum(1 for e in b if e) for b in basis)
-        flops = F * nq * (2 * 5 * 2 * (K + g) + 2 * 4 * K + 358)
+        flops = F * nq * (2 * 5 * 2 * FMAS_EVAL[K] + 15 + FLOPS_FLUX_PER_QP)
+        pipe = F * nq * (15 + FLOPS_FLUX_PER_QP)  # the two sides' gradients are added in FP64
         alg = F * (nq * 6 * w + 3 * w + 4 + 2 * 4 + 5 * w) + N * (K + 1) * 5 * w
         row = (((K + 1) * 5 + 3) // 4 * 4) * 4 if w == 4 else (K + 1) * 5 * w  # mixed: 16-byte rows
         layout = F * (nq * 10 * w + w + 2 * 4 + 5 * w) + N * row
     else:
-        cen = 5 * (2 * K * m.Mc + m.Mc)
-        dirf = 5 * 2 * (2 * m.nd * kd * m.Md + m.nd * m.Md) + 5 * 2 * (K * K + m.nd * kd * kd) + 5 * 60
-        flops = N * (cen + (dirf if m.nd else 0) + 5 * 2 * K)
+        cen = 2 * K * m.Mc + m.Mc
+        dirf = 2 * m.nd * kd * m.Md + m.nd * m.Md
+        left = 2 * K + (2 * K + 2 * m.nd * kd * kd + 60 if m.nd else 0)  # FP64 operations of the FP64 form
+        forms = 2 * (K * K + m.nd * kd * kd) + 60 if m.nd else 0
+        flops = N * 5 * (cen + dirf + forms + 2 * K)
+        pipe = N * 5 * left
         alg = N * (K * m.Mc * w + m.Mc * 4 + m.nd * (kd * m.Md * w + m.Md * 4) + (K * (K + 1) // 2) * w * (m.nd > 0)
                    + (K - 3) * w + w + 5 * 8 + (K + 1) * 5 * w)
         layout = alg
-    return {"flops": flops, "alg": alg, "layout": layout}
+    return {"flops": flops, "pipe_flops": pipe if w == 8 else flops, "alg": alg, "layout": layout}
 
 
 def roofline(m, prof: dict, form: str, peaks: dict, workload_key: str, frac_dir: float = 1.0) -> dict:
@@ -418,9 +420,9 @@ def roofline(m, prof: dict, form: str, peaks: dict, workload_key: str, frac_dir:
         name = "k_recon_mx<2,false,nd,gated>"
     alu_peak = peaks["fp32"] if mixed else peaks["fp64"]
     alu_src = ("FP32 FMA microbenchmark (ucns_alu_peak), of measured" if mixed
-               else "FP64 FMA microbenchmark (ucns_alu_peak), of measured; the contractions and polynomial "
-                    "evaluations run on the integer pipe, so the fraction is not bounded by 1")
-    alu = a["flops"] / avg_s / 1e12
+               else "FP64 FMA microbenchmark (ucns_alu_peak), of measured; operations left on the FP64 pipe "
+                    "(contractions and polynomial evaluations run on the integer pipe)")
+    alu = a["pipe_flops"] / avg_s / 1e12
     bw = a["alg"] / avg_s / 1e9
     alu_frac, hbm_frac = alu / alu_peak, bw / peaks["hbm"]
     if alu_frac >= hbm_frac:
@@ -431,6 +433,7 @@ def roofline(m, prof: dict, form: str, peaks: dict, workload_key: str, frac_dir:
                 "peak_source": peaks["hbm_source"]}
     roof.update({"kernel": name, "traffic": measured_traffic(name, f"{workload_key}/{form}"),
                  "avg_launch_ms": avg_s * 1e3, "algorithmic_flops_per_launch": a["flops"],
+                 "pipe_flops_per_launch": a["pipe_flops"],
                  "algorithmic_bytes_per_launch": a["alg"], "layout_bytes_per_launch": a["layout"],
                  "alu_frac": alu_frac, "hbm_frac": hbm_frac,
                  "hbm_frac_layout_bytes": a["layout"] / avg_s / 1e9 / peaks["hbm"]})

@@ -39,15 +39,33 @@ def test_p2_recon_bytes_gated_and_full():
 
 
 def test_ho_mixed_recon_bytes_are_the_tile_records():
-    # floats per 64-cell tile with CWENOZ (central chunks, smoothness matrix,
+    # floats per 32-cell tile with CWENOZ (central chunks, smoothness matrix,
     # directional chunks), as the library lays them out
-    tiles = {3: 19 * (2 * 64 + 19 * 2 * 64) + 190 * 64 + 6 * (6 * 64 + 3 * 6 * 64),
-             4: 17 * (4 * 64 + 34 * 4 * 64) + 595 * 64 + 18 * (6 * 64 + 9 * 6 * 64)}
+    tiles = {3: 19 * (2 * 32 + 19 * 2 * 32) + 190 * 32 + 6 * (6 * 32 + 3 * 6 * 32),
+             4: 17 * (4 * 32 + 34 * 4 * 32) + 595 * 32 + 18 * (6 * 32 + 9 * 6 * 32)}
     for order, (K, Mc, Md) in {3: (19, 38, 6), 4: (34, 68, 18)}.items():
-        m = _mesh(K, Mc, 6, Md, order * order, N=64)
+        m = _mesh(K, Mc, 6, Md, order * order, N=32)
         a = bench.algorithmic(m, "recon", mixed=True)
         rest = (K - 3) * 4 + 4 + 5 * 8 + (K + 1) * 5 * 4  # monomial means, 1/h, state, coefficients
         assert a["alg"] - m.n_cells * rest == tiles[order] * 4
+
+
+def test_ho_recon_flops_contract_the_directional_stencils_once():
+    # per variable: central members' differences and K rows over them, the same of six
+    # candidates, a^T M a of K and six times Kd modes, weights 60, scaling 2 K
+    for K, Mc, kd, Md in ((19, 38, 3, 6), (34, 68, 9, 18)):
+        m = _mesh(K, Mc, 6, Md, 9)
+        per = Mc * (1 + 2 * K) + 6 * Md * (1 + 2 * kd) + 2 * (K * K + 6 * kd * kd) + 60 + 2 * K
+        assert bench.algorithmic(m, "recon", mixed=True)["flops"] == m.n_cells * 5 * per
+        assert bench.algorithmic(m, "recon", mixed=False)["flops"] == m.n_cells * 5 * per
+
+
+def test_fp64_roofline_counts_the_operations_left_on_its_pipe():
+    for m in (_mesh(9, 18, 6, 6, 4), _mesh(19, 38, 6, 6, 9), _mesh(34, 68, 6, 18, 16)):
+        for kind in ("face", "recon"):
+            a, b = bench.algorithmic(m, kind, mixed=False), bench.algorithmic(m, kind, mixed=True)
+            assert 0 < a["pipe_flops"] < 0.6 * a["flops"]
+            assert b["pipe_flops"] == b["flops"] == a["flops"]
 
 
 def test_roofline_names_the_kernel_that_ran():
