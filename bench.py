@@ -330,7 +330,8 @@ def algorithmic(m, kind: str, mixed: bool, frac_dir: float = 1.0) -> dict:
     flops: as counted above; pipe_flops: those on the pipe that the roofline
     compares them with (in the FP64 form from P2 on the contractions, the P3/P4
     smoothness rows and the polynomial evaluations run on the integer pipe).
-    bytes: each array element the kernel needs crossing HBM once (neighbour gathers served by cache), in two countings:
+    bytes: each array element the kernel needs crossing HBM once (neighbour
+    gathers served by cache), in two countings:
       "alg": the minimal data -- per Gauss point its position relative to the
         owner's centroid and its area vector (6 words), per face the offset
         between the two centroids (3 words), the penalty factor, two cell ids

@@ -316,7 +316,8 @@ __global__ void __launch_bounds__(256) k_recon_p1(ReconArgs a) {
 // loads' latency at 12 warps per SM), from shared memory tiles 1648, with the
 // differences in integers too and one division for all weights 1192 (3, 4, 5
 // blocks per SM: 1210, 1192, 1229), with single-instruction accumulation and
-// coefficients written in fixed point 1060.
+// coefficients written in fixed point 1067, and 1081 since differences are rounded
+// after their shift down (54 a thread).
 template <bool WENO, int ND, bool GATED, bool WALLS = false>
 __global__ void __launch_bounds__(FxTile::THREADS, 4) k_recon(ReconArgs a) {
   using T = FxTile;
@@ -569,7 +570,8 @@ struct FxPoint {
   }
 };
 
-// both sides' values and the sum of their gradients; nb < 0: the owner's values and gradients alone
+// both sides' values and the sum of their gradients; nb < 0 (a boundary face): the owner's
+// polynomial at its centroid in place of the other side's, for the caller to replace
 template <int ORDER>
 __device__ __forceinline__ void eval_sides(const FaceArgs& a, int o, int nb, const int2* __restrict__ fx, size_t F,
                                            double UL[5], double UR[5], double gs[5][3]) {

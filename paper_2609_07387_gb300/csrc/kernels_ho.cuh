@@ -10,8 +10,8 @@
 //   k_face_ho   ORDER^2 Gauss points per face on ORDER^2 lanes (9 at P3, 16
 //               at P4; 32 / ORDER^2 faces per warp); values and gradients of
 //               the monomial-form polynomials, HLLC, penalised viscous flux
-//               (Eq. 7), and the face total summed by the group's first lane
-//               over its lanes in point order (deterministic).
+//               (Eq. 7), and each (face, variable) total summed by a lane of
+//               its own in point order (deterministic).
 //   k_recon_ho_mx the same in the mixed form, tile by tile (32 cells): the
 //               stencil ids and FP32 pseudo-inverses stream through shared
 //               memory in bulk-copied chunks, thread = (cell, variable).
@@ -102,9 +102,9 @@ __device__ __forceinline__ double si_form(const double* __restrict__ M, size_t N
 // warp that streams the tile's chunks through a ring of S shared-memory stages, every
 // wait bounded.  The differences of a stencil wait in shared memory as operands while
 // its rows pass; the central coefficients (xi units) wait in the output array.
-// Bound by latency at two warps per scheduler (issue 30 %, FP64 pipe 25 %): 11
+// Bound by latency at two warps per scheduler (P4: issue 28 %, FP64 pipe 42 %): 11
 // thousand integer multiply-adds a thread at P4.  P4 CWENOZ at 24^3, us: FP64
-// contractions from global memory 852, this 339 (418 with the directional
+// contractions from global memory 852, this 329 (418 with the directional
 // contractions run twice and the row exponents read from global memory).
 template <int ORDER, bool WENO>
 __global__ void __launch_bounds__(HOFxTile<ORDER>::THREADS, 2) k_recon_ho(ReconArgsHO a) {
@@ -363,7 +363,7 @@ __global__ void __launch_bounds__(HOFxTile<ORDER>::THREADS, 2) k_recon_ho(ReconA
 // in shared memory, one column per thread, for the flux.  Bound by the FP64 pipe and
 // its latency.  P4 at 24^3, us: evaluation in FP64 1635, in integers unrolled 969
 // (8 warps per SM), in this loop 548 (6, 8, 10 blocks per SM: 637, 548, 595), the
-// constant term added as an integer 534.
+// constant term added as an integer 534, with the face sums shared out 453.
 constexpr int kFaceHoThreads = 64;
 template <int ORDER, bool VISC>
 __global__ void __launch_bounds__(kFaceHoThreads, 8) k_face_ho(FaceArgs a) {
@@ -434,7 +434,7 @@ __global__ void __launch_bounds__(kFaceHoThreads, 8) k_face_ho(FaceArgs a) {
 // stencil differences from the float pairs of the FP64 state, FP32
 // pseudo-inverses, contractions, smoothness forms and weights; the constant
 // term written relative to the reference state U_ref; coefficients FP32
-// [K+1][N][5]; FP32 HLLC and viscous flux on reference-relative states, FP32
+// rows [N][cs]; FP32 HLLC and viscous flux on reference-relative states, FP32
 // face totals (k_rk<s, nfc, float> sums them as float pairs into FP64).
 struct ReconArgsHOMx {
   const float* __restrict__ Uhl;    // [N][5][2] float pairs (hi, lo) of the state
