@@ -1,6 +1,7 @@
 """The fixed-point sums of csrc/fixed.cuh on the host, against exact rational
-arithmetic: differences, contractions and conversions of FP64 values of one
-magnitude, of mixed ones, subnormal and near the largest, and non-finite ones.
+arithmetic: differences, contractions, polynomial coefficients and conversions
+of FP64 values of one magnitude, spread over many binades, at and beside powers
+of two, subnormal and near the largest, and non-finite ones.
 The bounds are those of the header: a sum is off by at most (2^-57 + M 2^-56.5)
 sum|P| max|u_m - u_0| and the final rounding."""
 import os
