@@ -550,15 +550,18 @@ __device__ __forceinline__ void hllc_flux_mx(const float WL[5], const float WR[5
   // 0), written without branches: the side's quantities are selected first, and
   // outside the star region (S_L >= 0 on the left, S_R < 0 on the right) the star
   // speed is taken as the side's own u_n, where the star flux is the physical
-  // flux.  With s the star speed and r* = (s - u_n)/(S - s): rho* = rho (1 + r*);
-  // momentum with p' (the dropped p_ref n integrates to zero), energy s (E* + p*) =
-  // s (E + p)(1 + r*) + s (s - u_n)(rho* s + m), E + p = H_ref + E' + p'.  The large
-  // parts rho s and H_ref s are rounded once, as in a plain flux.
+  // flux (and m = rho (S - u_n) as 0: a side whose wave speed is NaN, as beside a
+  // negative pressure, counts as outside).  With s the star speed and r* = (s -
+  // u_n)/(S - s): rho* = rho (1 + r*); momentum with p' (the dropped p_ref n integrates
+  // to zero), energy s (E* + p*) = s (E + p)(1 + r*) + s (s - u_n)(rho* s + m), E + p =
+  // H_ref + E' + p'.  The large parts rho s and H_ref s are rounded once, as in a plain
+  // flux.
   const bool left = 0.f <= SL || 0.f <= Ss;
   const float r = left ? rL : rR, un = left ? unL : unR, pp = left ? ppL : ppR;
-  const float S = left ? SL : SR, m = left ? mL : mR;
+  const float S = left ? SL : SR;
   const float hp = (left ? WL[4] : WR[4]) + pp;
   const bool in_star = left ? SL < 0.f : 0.f <= SR;
+  const float m = in_star ? r * (S - un) : 0.f;
   const float s = in_star ? Ss : un;
   const float ds = s - un;
   const float rs = in_star ? fdiv(ds, S - s) : 0.f;
